@@ -139,7 +139,11 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace,
  * stream, phi = sum g (Eq. 35), psi (Eq. 37, phi clipped to [0,1]),
  * isotropic stencils (Sec. 3.2), hbar (Eq. 2), F = hbar grad phi, u and p
  * (Eqs. 28-29), MRT collision of f (Eqs. 21-25) and of g (Eqs. 31-33) with
- * d_t(phi u) by backward difference.  Asynchronous on the handle's stream:
+ * d_t(phi u) by backward difference.  Asynchronous on the handle's stream.
+ * Batches that fit the SMs' shared memory (about 150,000 nodes in FP32,
+ * 75,000 in FP64) run 4 steps or more as cooperative launches of up to 1,024
+ * steps that keep the state on the chip, unless another kernel was asked for,
+ * volumes are tracked or the stream is being captured.  Otherwise
  * runs of 4 steps or more are cut into chunks of up to 64 steps; the first
  * chunk of a given length (and source buffer) is launched directly, and
  * when that length comes again its steps are captured into a CUDA graph,
@@ -185,7 +189,8 @@ int lbm_set_row_chains(lbm_handle* h, int32_t on);
 int32_t lbm_get_row_chains(const lbm_handle* h);
 
 /* Bound of the device waits, in SM clock cycles: the bulk-copy kernel's
- * waits for its staged rows and the persistent kernel's grid barrier.  A
+ * waits for its staged rows, the chip-resident kernel's waits for its
+ * neighbours' rims and the persistent kernel's grid barrier.  A
  * wait that gives up raises LBM_ERR_TIMEOUT (reported by the next
  * synchronising call or lbm_status); the kernel first waits, with the
  * default bound, for the copies it issued, then returns, and the step's
@@ -258,9 +263,12 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel,
 
 /* Step-kernel variant: 0 = automatic, 1 = register-pipelined loads (any
  * grid), 2 = bulk-copy (TMA) staged loads through shared memory (needs every
- * case to have nx >= 4 and nx a multiple of 4 in FP32, of 2 in FP64).  Both
- * run the same per-node arithmetic (equal up to rounding, see
- * lbm_set_tiling).  lbm_get_kernel returns the variant in use (1 or 2).
+ * case to have nx >= 4 and nx a multiple of 4 in FP32, of 2 in FP64), 3 = one
+ * cooperative launch for many steps (at most 4 Mi nodes; the chip-resident
+ * kernel where the batch fits it, see lbm_step, else a grid barrier between
+ * steps).  All run the same per-node arithmetic (equal up to rounding, see
+ * lbm_set_tiling).  lbm_get_kernel returns the variant of single steps in use
+ * (1 or 2, or 3 if asked for).
  * Changing the variant rebuilds the work-item table (whole-row chains run
  * the bulk-copy kernel only; synchronises). */
 int lbm_set_kernel(lbm_handle* h, int32_t variant);

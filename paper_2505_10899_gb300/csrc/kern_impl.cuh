@@ -7,6 +7,7 @@
 #include "lbm_aux.cuh"
 #include "lbm_kernels.cuh"
 #include "lbm_kernels_tma.cuh"
+#include "lbm_resident.cuh"
 
 namespace lbmk {
 
@@ -123,6 +124,55 @@ cudaError_t launch_persistent<LBM_T>(const StepArgs<LBM_T>& a, int bx, bool coup
                              : persist_bx<128, false>(a, n_items, nsteps, flip, count, gen, s);
     default: return cudaErrorInvalidValue;
   }
+}
+
+template <bool COUPLED, int V>
+struct ResKernel {
+  static constexpr ResVariant X = res_variant(sizeof(LBM_T) == 8, COUPLED, V);
+  static constexpr size_t BYTES = ResShape<LBM_T, COUPLED, X.pc, X.nx>::SMEM_BYTES;
+  static_assert(X.per_sm * (BYTES + 1280) <= 228 * 1024, "shared memory of an SM");
+  static const void* fn() {
+    return (const void*)step_resident<LBM_T, COUPLED, X.nt, X.r, X.pc, X.nx, X.per_sm>;
+  }
+};
+
+template <typename F>
+cudaError_t res_pick(bool coupled, int v, F&& f) {
+  switch (v) {
+    case 0: return coupled ? f(ResKernel<true, 0>()) : f(ResKernel<false, 0>());
+    case 1: return coupled ? f(ResKernel<true, 1>()) : f(ResKernel<false, 1>());
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+template <>
+cudaError_t launch_resident<LBM_T>(const StepArgs<LBM_T>& a, bool coupled, int variant,
+                                   const ResTile* tiles, int ntiles, const ResRun& run,
+                                   cudaStream_t s) {
+  return res_pick(coupled, variant, [&](auto k) {
+    StepArgs<LBM_T> args = a;
+    ResRun r = run;
+    void* params[] = {(void*)&args, (void*)&tiles, (void*)&r};
+    return cudaLaunchCooperativeKernel(decltype(k)::fn(), dim3(ntiles), dim3(decltype(k)::X.nt),
+                                       params, decltype(k)::BYTES, s);
+  });
+}
+
+template <>
+bool resident_fits<LBM_T>(bool coupled, int variant, int ntiles) {
+  int dev = 0, nsm = 0, per_sm = 0;
+  const cudaError_t e = res_pick(coupled, variant, [&](auto k) -> cudaError_t {
+    using KX = decltype(k);
+    cudaError_t r = cudaFuncSetAttribute(KX::fn(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)KX::BYTES);
+    if (r == cudaSuccess) r = cudaGetDevice(&dev);
+    if (r == cudaSuccess) r = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (r == cudaSuccess)
+      r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, KX::fn(), KX::X.nt, KX::BYTES);
+    return r;
+  });
+  if (e != cudaSuccess) cudaGetLastError();  // not available: the other kernels run
+  return e == cudaSuccess && (int64_t)per_sm * nsm >= ntiles;
 }
 
 template <>

@@ -29,6 +29,41 @@ cudaError_t launch_persistent(const StepArgs<T>& a, int bx, bool coupled, int n_
                               int nsteps, int flip, unsigned int* count, unsigned int* gen,
                               cudaStream_t s);
 
+// Variants of the chip-resident kernel: nt threads per CTA with r nodes each,
+// pc cells of shared memory (nodes and their two-node surround), nx rim
+// triples at most, per_sm CTAs per SM.  The first that holds a batch runs it.
+// Measured, us per step over 256 steps:
+//   FP32 coupled     128x64  256x128  384x192  512x256
+//   256 x 1, 2/SM     1.68     2.05      -        -     (more CTAs: rims overlap)
+//   512 x 1, 1/SM     1.71     2.18      -        -
+//   512 x 2, 1/SM     1.77     2.24     2.60     3.73
+//   448 x 2, 1/SM     1.73     2.23     2.97     4.26
+//   896 x 1, 1/SM     1.85     2.34     2.73     4.02   (72 registers)
+// The vortex holds twice the nodes (g alone): 256^2 2.31 with 512 x 1, 512^2
+// 4.28 with 896 x 2.  FP64 is bound by its pipe (128x64: 14.2, 256x128: 26.5);
+// spare threads change nothing there.
+struct ResVariant {
+  int nt, r, pc, nx, per_sm;
+};
+constexpr int kResVariants = 2;
+constexpr ResVariant kRes32[kResVariants] = {{256, 1, 448, 384, 2}, {512, 2, 1296, 640, 1}};
+constexpr ResVariant kRes64[kResVariants] = {{256, 1, 448, 384, 1}, {256, 2, 704, 512, 1}};
+constexpr ResVariant kRes32V[kResVariants] = {{512, 1, 784, 512, 1}, {896, 2, 2304, 768, 1}};
+constexpr ResVariant kRes64V[kResVariants] = {{512, 1, 784, 512, 1}, {512, 2, 1296, 768, 1}};
+constexpr ResVariant res_variant(bool f64, bool coupled, int v) {
+  return coupled ? (f64 ? kRes64[v] : kRes32[v]) : (f64 ? kRes64V[v] : kRes32V[v]);
+}
+
+// Chip-resident kernel (cooperative launch of ntiles CTAs).
+template <typename T>
+cudaError_t launch_resident(const StepArgs<T>& a, bool coupled, int variant,
+                            const ResTile* tiles, int ntiles, const ResRun& run, cudaStream_t s);
+
+// Whether ntiles CTAs of a variant are co-resident on the current device
+// (also allows the variant's dynamic shared memory; before the first launch).
+template <typename T>
+bool resident_fits(bool coupled, int variant, int ntiles);
+
 // Allow the dynamic shared memory of every TMA kernel variant on the current
 // device (call once per device before the first launch or graph capture).
 template <typename T>

@@ -244,7 +244,8 @@ int max_items(const lbm_params* c, int n) {
   return (int)std::min<int64_t>(m, INT32_MAX);
 }
 
-Layout make_layout(const lbm_params* c, int n, int n_items, int total_regions) {
+Layout make_layout(const lbm_params* c, int n, int n_items, int total_regions,
+                   const lbmk::ResPlan& res) {
   Layout L;
   const size_t es = elem_size(c[0].precision);
   const bool coupled = c[0].flow == LBM_FLOW_COUPLED;
@@ -263,6 +264,11 @@ Layout make_layout(const lbm_params* c, int n, int n_items, int total_regions) {
   off = align_up(off + (size_t)n * sizeof(lbmk::InitSrc));
   L.chainc = off;  // case indices, chain by chain
   off = align_up(off + (size_t)n * sizeof(int));
+  L.rtiles = off;  // chip-resident kernel: tiles, two sets of exchange slots
+  off = align_up(off + res.tiles.size() * sizeof(lbmk::ResTile));
+  L.rslots = off;
+  L.rslot_bytes = (size_t)2 * res.nslots * 16 * (es == 8 ? 3 : 1);
+  off = align_up(off + L.rslot_bytes);
   int64_t maxp = 0;
   for (int k = 0; k < n; ++k) maxp = std::max<int64_t>(maxp, (int64_t)c[k].nx * c[k].ny);
   L.staging = off;
@@ -441,6 +447,64 @@ int launch_persist(lbm_handle* h, cudaStream_t s, int parity, int nsteps, int fl
     e = lbmk::launch_persistent<double>(step_args<double>(h, parity, 0), h->tile.bx, coupled, n,
                                         nsteps, flip, bar_count(h), bar_gen(h), s);
   if (e != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("persistent launch: ") + cudaGetErrorString(e));
+  return LBM_OK;
+}
+
+// Whether a run of nsteps steps takes the chip-resident kernel: the batch
+// fits, no other kernel was asked for, no per-step volumes are tracked, and
+// the stream is not being captured (a replayed launch would reuse its tags).
+constexpr int64_t kResMinSteps = 4;
+bool use_resident(const lbm_handle* h, int64_t nsteps) {
+  if (h->res.variant < 0 || h->track || (h->kernel != 0 && h->kernel != 3) ||
+      nsteps < (h->kernel == 3 ? 1 : kResMinSteps))
+    return false;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+    cudaGetLastError();  // another stream's capture forbids the query
+    return false;
+  }
+  return st == cudaStreamCaptureStatusNone;
+}
+
+// nsteps (at most kResMaxSteps) steps in one launch of the chip-resident
+// kernel.  store = false: the state is left as it is (autotuning trials).
+// rec: the states entering each step are recorded, `stride` bytes apart.
+template <typename T>
+int launch_res(lbm_handle* h, int nsteps, bool store, void* rec, int64_t stride) {
+  if (h->res_epoch > UINT32_MAX - 2 * lbmk::kResMaxSteps) {  // tags run out: start over
+    LBM_CUDA(cudaMemsetAsync(h->ws + h->L.rslots, 0, h->L.rslot_bytes, h->stream));
+    h->res_epoch = 1;
+  }
+  lbmk::ResRun r{};
+  r.nsteps = nsteps;
+  r.store = store ? 1 : 0;
+  r.epoch = h->res_epoch;
+  r.nslots = h->res.nslots;
+  r.slots = h->ws + h->L.rslots;
+  r.t0 = h->t;
+  r.t_dev = h->t_dev;
+  r.rec = rec;
+  r.rec_stride = stride / (int64_t)sizeof(T);
+  h->res_epoch += (uint32_t)nsteps;
+  const cudaError_t e = lbmk::launch_resident<T>(
+      step_args<T>(h, h->parity, 0), h->flow == LBM_FLOW_COUPLED, h->res.variant,
+      (const lbmk::ResTile*)(h->ws + h->L.rtiles), (int)h->res.tiles.size(), r, h->stream);
+  if (e != cudaSuccess)
+    return fail(LBM_ERR_CUDA, std::string("resident launch: ") + cudaGetErrorString(e));
+  return LBM_OK;
+}
+
+int run_resident(lbm_handle* h, int64_t nsteps, void* rec = nullptr, int64_t stride = 0) {
+  while (nsteps > 0) {
+    const int cnt = (int)std::min<int64_t>(nsteps, lbmk::kResMaxSteps);
+    const int rc = h->precision == LBM_F32 ? launch_res<float>(h, cnt, true, rec, stride)
+                                           : launch_res<double>(h, cnt, true, rec, stride);
+    if (rc) return rc;
+    if (rec) rec = (char*)rec + cnt * stride;
+    h->parity ^= (cnt & 1);
+    h->t += cnt;
+    nsteps -= cnt;
+  }
   return LBM_OK;
 }
 
@@ -774,7 +838,9 @@ const char* lbm_status_string(int s) {
 
 size_t lbm_workspace_bytes(const lbm_params* cases, int32_t ncases) {
   if (check_params(cases, ncases) != LBM_OK) return 0;
-  return make_layout(cases, ncases, max_items(cases, ncases), ncases * lbmk::kMaxRegions).total;
+  return make_layout(cases, ncases, max_items(cases, ncases), ncases * lbmk::kMaxRegions,
+                     lbmk::res_plan(cases, ncases))
+      .total;
 }
 
 int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t ws_bytes,
@@ -803,7 +869,8 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t 
   h->vol_base.resize(ncases);
   for (int k = 0; k < ncases; ++k) h->vol_base[k] = k;
   h->total_regions = ncases;
-  h->L = make_layout(cases, ncases, max_items(cases, ncases), ncases * lbmk::kMaxRegions);
+  h->res = lbmk::res_plan(cases, ncases);
+  h->L = make_layout(cases, ncases, max_items(cases, ncases), ncases * lbmk::kMaxRegions, h->res);
   if (ws_bytes < h->L.total) {
     const size_t need = h->L.total;
     delete h;
@@ -857,6 +924,18 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t 
   }
   if (cudaMemsetAsync(h->ws + h->L.hdr, 0, 64, h->stream) != cudaSuccess)
     return cleanup(fail(LBM_ERR_CUDA, "header upload failed"));
+  if (h->res.variant >= 0) {
+    const bool coupled = h->flow == LBM_FLOW_COUPLED;
+    const int nt = (int)h->res.tiles.size();
+    if (!(h->precision == LBM_F32 ? lbmk::resident_fits<float>(coupled, h->res.variant, nt)
+                                  : lbmk::resident_fits<double>(coupled, h->res.variant, nt)))
+      h->res.variant = -1;
+    else if (cudaMemcpyAsync(h->ws + h->L.rtiles, h->res.tiles.data(),
+                             nt * sizeof(lbmk::ResTile), cudaMemcpyHostToDevice,
+                             h->stream) != cudaSuccess ||
+             cudaMemsetAsync(h->ws + h->L.rslots, 0, h->L.rslot_bytes, h->stream) != cudaSuccess)
+      return cleanup(fail(LBM_ERR_CUDA, "tile upload failed"));
+  }
   // items, chains and cases; labels planes: zero (region 0 everywhere)
   // until lbm_set_regions
   rc = upload_plan(h);
@@ -940,6 +1019,7 @@ int lbm_step(lbm_handle* h, int64_t nsteps) {
   lbmk::TraceRange trace("lbm_step");
   if (!h) return fail(LBM_ERR_ARG, "null handle");
   if (nsteps < 0) return fail(LBM_ERR_ARG, "nsteps < 0");
+  if (use_resident(h, nsteps)) return run_resident(h, nsteps);
   if (h->kernel == 3 && !h->track) {
     // persistent kernel: chunks of at most 65536 steps per cooperative launch
     while (nsteps > 0) {
@@ -991,6 +1071,7 @@ int lbm_prepare_steps(lbm_handle* h, int64_t nsteps) {
   if (nsteps < 0) return fail(LBM_ERR_ARG, "nsteps < 0");
   if (h->kernel == 3 && !h->track) return LBM_OK;  // one cooperative launch, nothing to capture
   if (nsteps < kDirectSteps) return LBM_OK;         // launched directly
+  if (use_resident(h, nsteps)) return LBM_OK;       // one cooperative launch
   int parity = h->parity;
   while (nsteps > 0) {
     const int cnt = (int)std::min<int64_t>(nsteps, kGraphSteps);
@@ -1097,8 +1178,21 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
           h->row_chains = rcv == 1;
           rc = lbm_set_tiling(h, bx, rows);
           if (rc != LBM_OK) break;
+          int n_run = n_trial;
           cudaError_t e = cudaSuccess;
-          if (kv == 3) {  // one launch of n_trial steps without flipping buffers
+          if (kv == 3 && h->res.variant >= 0) {
+            // the chip-resident kernel has tiles of its own: one trial
+            if (bx != 128 || rows != 2) continue;
+            n_run = std::max(n_trial, kGraphSteps);
+            auto trial = [&]() {
+              return h->precision == LBM_F32 ? launch_res<float>(h, n_run, false, nullptr, 0)
+                                             : launch_res<double>(h, n_run, false, nullptr, 0);
+            };
+            rc = trial();
+            if (rc == LBM_OK) e = cudaEventRecord(e0, h->stream);
+            if (rc == LBM_OK && e == cudaSuccess) rc = trial();
+            if (rc != LBM_OK) break;
+          } else if (kv == 3) {  // one launch of n_trial steps without flipping buffers
             rc = launch_persist(h, h->stream, h->parity, 1, 0);
             if (rc == LBM_OK) e = cudaEventRecord(e0, h->stream);
             if (rc == LBM_OK && e == cudaSuccess) rc = launch_persist(h, h->stream, h->parity, n_trial, 0);
@@ -1122,10 +1216,11 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
             rc = fail(LBM_ERR_CUDA, std::string("autotune: ") + cudaGetErrorString(e));
             break;
           }
-          if (ms / n_trial < best) {
-            best = ms / n_trial;
+          if (ms / n_run < best) {
+            best = ms / n_run;
             best_t.bx = bx;
             best_t.rows = rows;
+            if (kv == 3 && h->res.variant >= 0) best_t = keep_tile;
             best_k = kv;
             best_rc = rcv == 1;
           }
@@ -1435,6 +1530,9 @@ int lbm_record_steps(lbm_handle* h, int64_t count, void* d_states, int64_t strid
   if (count < 0) return fail(LBM_ERR_ARG, "count < 0");
   if (count > 1 && stride_bytes < (int64_t)lbm_snapshot_bytes(h, 0))
     return fail(LBM_ERR_ARG, "stride_bytes smaller than a snapshot");
+  // the chip-resident kernel writes the states as it goes
+  if (stride_bytes % (int64_t)elem_size(h->precision) == 0 && use_resident(h, count))
+    return run_resident(h, count, d_states, stride_bytes);
   for (int64_t j = 0; j < count; ++j) {
     int rc = lbm_snapshot(h, 0, (char*)d_states + j * stride_bytes);
     if (rc) return rc;

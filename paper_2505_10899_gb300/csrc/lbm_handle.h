@@ -10,11 +10,13 @@
 
 #include "../../include/lbm_api.h"
 #include "lbm_layout.h"
+#include "lbm_res_plan.h"
 
 namespace lbmk {
 
 struct Layout {
   size_t hdr = 0, cases = 0, items = 0, part = 0, vol = 0, init = 0, chainc = 0, staging = 0;
+  size_t rtiles = 0, rslots = 0, rslot_bytes = 0;  // chip-resident kernel
   std::vector<size_t> f, g, J, lab;  // per-case offsets (f: 2 buffers back to back)
   std::vector<size_t> glo;           // FP32: low part of g_0, 2 planes per case
   std::vector<int64_t> plane;
@@ -88,6 +90,10 @@ struct lbm_handle {
   double* vol = nullptr;
   double* staging = nullptr;
   int64_t max_plane = 0;
+  // chip-resident kernel: tiles (none if the batch does not fit), and the tag
+  // of its next exchange
+  lbmk::ResPlan res;
+  uint32_t res_epoch = 1;
   // reverse mode (lbm_adjoint_attach): caller-provided FP64 scratch
   char* adj_ws = nullptr;
   size_t adj_ws_bytes = 0;

@@ -82,6 +82,31 @@ struct InitSrc {
 };
 
 
+// One tile of the chip-resident kernel (lbm_resident.cuh): nodes
+// [x0, x0 + w) x [y0, y0 + h) of case c.  hS, hN: heights of the tile rows
+// below and above.  slot, nb: first exchange slot of the tile and of its
+// neighbours (beyond a wall: unused).
+enum { kResW = 0, kResE = 3, kResS = 6, kResN = 7 };  // W, SW, NW; E, SE, NE; S; N
+struct ResTile {
+  int32_t c, x0, y0, w, h, hS, hN;
+  uint32_t slot;
+  uint32_t nb[8];
+};
+constexpr int kResMaxSteps = 1024;  // steps of one launch
+
+// One launch of the chip-resident kernel.
+struct ResRun {
+  int32_t nsteps;      // 1 .. kResMaxSteps
+  int32_t store;       // 0: leave the state as it is (autotuning trials)
+  uint32_t epoch;      // tag of the first exchange, unique over the handle's launches
+  uint32_t nslots;     // exchange slots of one set (two sets)
+  void* slots;
+  int64_t t0;          // step index at the start
+  int64_t* t_dev;      // device step clock, advanced at the end
+  void* rec;           // record S_t0 .. S_{t0+nsteps-1} (lbm_snapshot layout), or null
+  int64_t rec_stride;  // elements between recorded states
+};
+
 enum { kModeStep = 0, kModeFields = 1 };
 enum { kFlagNonFinite = 1, kFlagTimeout = 2 };
 
