@@ -274,12 +274,19 @@ int lbm3_init(const lbm3_params* p, void* d_ws, size_t ws_bytes, const double* h
   h->vol = reinterpret_cast<double*>(h->ws + c.vol);
   h->staging = reinterpret_cast<double*>(h->ws + c.staging);
   h->hp = host_params(*p, c.plane);
-  // default tiling: 32 x 8 columns, zc planes such that a step has about
-  // 8 CTAs per SM
-  const int64_t cols = lbmk3::n_ctas(p->nx, p->ny, 1, 32, 8, 1);
-  int zc = (int)std::max<int64_t>(1, cols * p->nz / (152 * 8));
-  zc = std::max(zc_min(*p), std::min(zc, 64));
-  h->bx = 32, h->by = 8, h->zc = std::min(zc, p->nz);
+  // Default tiling: 32 x 4 columns (128 threads, four CTAs per SM at 128
+  // registers; the 256 threads of 32 x 8 make two, and lose a fifth: us per
+  // step in FP32, 32 x 8 -> 32 x 4: 90 x 75 x 66 30.3 -> 25.6, 150^3 231 ->
+  // 193, 256 x 256 x 128 505 -> 410).  Planes: a CTA takes about zc + 2 plane
+  // times (its first two phi planes), a step as many as it has waves of CTAs.
+  h->bx = 32, h->by = 4;
+  double best = 1e300;
+  for (int zc : {8, 10, 12, 16, 20, 24, 32, 48, 64}) {
+    const int z = std::min(std::max(zc, zc_min(*p)), p->nz);
+    const double waves = (double)lbmk3::n_ctas(p->nx, p->ny, p->nz, 32, 4, z) / (152 * 4);
+    const double cost = (waves <= 3 ? std::ceil(waves) : waves + 0.5) * (z + 2.2);
+    if (cost < best) best = cost, h->zc = z;
+  }
   auto bail = [&](int code) {
     if (h->cap) cudaStreamDestroy(h->cap);
     delete h;

@@ -209,11 +209,20 @@ Plan make_plan(const lbm_params* c, int n, const Tiling& t, int nreq, bool rowmo
   return pl;
 }
 
-// Default tiling: the widest strip that leaves at most 15% of the threads idle
-// on ragged strips, and runs of 16 rows (short runs balance the load across
-// SMs; the halo rows they re-read come from L2) unless the batch is too small
-// to give every SM several CTAs.
-Tiling choose_tiling(const lbm_params* c, int n) {
+// Default tiling.  Strips: the widest that leaves at most 15% of the threads
+// idle on ragged strips (narrower ones only add halo columns: 237,000 nodes in
+// 8 cases run 19.1 us per step in 128 x 4, 21.6 in 64 x 4, 24.3 in 32 x 4).
+// Rows: a CTA of `rows` rows takes about rows + 2.5 row times in FP32 (the
+// halo rows and the prologue), and the step as many of these as it has waves
+// of resident CTAs: whole waves where one grid fills few of them, half a wave
+// of tail where there are many, or uneven cases and two chains.  Measured, us
+// per step (16 rows as the fixed choice -> this one): 1024^2 45.4 -> 42.8,
+// 2048^2 149 -> 134, 8192 x 4096 973 -> 964, 16 uneven cases 46.1 -> 39.0,
+// 512 cases 1173 -> 1144.  FP64 is bound by its pipe, which CTAs of one SM
+// share: the fullest SM decides, a halo row costs its phi and psi only, and
+// fewer than three CTAs per SM leave the pipe idle (2048^2 3045 -> 2967; 8
+// uneven cases of 237,000 nodes: 520 CTAs 209, 260 CTAs 236, 130 CTAs 272).
+Tiling choose_tiling(const lbm_params* c, int n, bool tma) {
   int64_t nodes = 0;
   for (int k = 0; k < n; ++k) nodes += (int64_t)c[k].nx * c[k].ny;
   Tiling t;
@@ -226,13 +235,22 @@ Tiling choose_tiling(const lbm_params* c, int n) {
       break;
     }
   }
-  const int64_t want = 152 * 12;  // CTAs for a full machine
-  int64_t rows = nodes / (t.bx * want);
-  while (rows < 4 && t.bx > 32) {
-    t.bx /= 2;
-    rows = nodes / (t.bx * want);
+  // CTAs of 128 threads per SM that the registers allow
+  const int slots = 152 * (128 / t.bx) * (tma ? 6 : 3);
+  double best = 1e300;
+  for (int rows : {2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64}) {
+    int64_t items = 0;
+    for (int k = 0; k < n; ++k)
+      items += (int64_t)((c[k].nx + t.bx - 1) / t.bx) * ((c[k].ny + rows - 1) / rows);
+    double cost;
+    if (c[0].precision == LBM_F64) {
+      cost = (double)std::max<int64_t>((items + 151) / 152, 3) * (rows + 0.6);
+    } else {
+      const double waves = (double)items / slots;
+      cost = (n == 1 && waves <= 4 ? std::ceil(waves) : std::max(1.0, waves + 0.5)) * (rows + 2.5);
+    }
+    if (cost < best) best = cost, t.rows = rows;
   }
-  t.rows = (int)std::max<int64_t>(2, std::min<int64_t>(16, rows));
   return t;
 }
 
@@ -863,7 +881,6 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t 
   h->precision = cases[0].precision;
   h->flow = cases[0].flow;
   h->stream = (cudaStream_t)stream;
-  h->tile = choose_tiling(cases, ncases);
   h->chains_req = std::min(2, ncases);
   h->nregions.assign(ncases, 1);
   h->vol_base.resize(ncases);
@@ -897,6 +914,7 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t 
     for (int k = 0; k < ncases; ++k)
       if (cases[k].walls) h->tma_ok = false;
   }
+  h->tile = choose_tiling(cases, ncases, h->tma_ok);
   h->chain_cases_dev = (int*)(h->ws + h->L.chainc);
   {
     Plan pl = make_plan(cases, ncases, h->tile, h->chains_req, rowmode(h));
