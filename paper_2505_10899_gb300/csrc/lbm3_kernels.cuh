@@ -31,6 +31,7 @@
 #include <cuda_runtime.h>
 
 #include "lbm3_layout.h"
+#include "lbm_math.cuh"
 
 namespace lbmk3 {
 
@@ -59,9 +60,11 @@ struct N3<float> {
 template <>
 struct N3<double> {
   using pair = double2;
-  static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-  static __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
-  static __device__ __forceinline__ double lratio(double a, double b) { return log(a / b); }
+  static __device__ __forceinline__ double rcp(double x) { return lbmk::rcp64(x); }
+  static __device__ __forceinline__ double rsq(double x) { return lbmk::rsq64(x); }
+  static __device__ __forceinline__ double lratio(double a, double b) {
+    return lbmk::lratio64(a, b);
+  }
   static __device__ __forceinline__ double clamp01(double v) { return fmin(fmax(v, 0.0), 1.0); }
 };
 

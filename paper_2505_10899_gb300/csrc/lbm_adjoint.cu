@@ -163,6 +163,8 @@ struct AdArgs {
 // which the normal of Eq. 17 does not see).
 template <typename R>
 __device__ __forceinline__ R dpsi_dphi(R p, R xi) {
+  if constexpr (sizeof(R) == 8)
+    return lbmk::rcp64(p + xi) + lbmk::rcp64((R(1) - p) + xi);
   const R d = R(1) / (p + xi) + R(1) / ((R(1) - p) + xi);
   return sizeof(R) == 4 ? R(1.4426950408889634) * d : d;
 }

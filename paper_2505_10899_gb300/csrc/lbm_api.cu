@@ -344,6 +344,9 @@ Phys<T> make_phys(const lbm_params& p) {
     ph.gsD[i] = (T)(-sg[i] * kD[i]);
     ph.ghD3[i] = (T)((1.0 - 0.5 * sg[i]) * kD[i] / 3.0);
   }
+  ph.unit = 1;
+  for (int i = 0; i < 9; ++i)
+    if ((i < 7 && p.s_f[i] != 1.0) || (i > 0 && i != 3 && i != 5 && p.s_g[i] != 1.0)) ph.unit = 0;
   ph.vU = p.vortex_U;
   ph.vT = p.vortex_T;
   return ph;

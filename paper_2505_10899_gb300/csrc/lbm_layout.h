@@ -64,6 +64,7 @@ struct Phys {
   T fsD[kQ], fhD[kQ];
   T gsD[kQ], ghD3[kQ];  // ghD3 = ghD / 3 (the source moments carry a 1/3)
   double vU, vT;        // prescribed vortex amplitude and period
+  int32_t unit;         // all free rates are 1 (FP64 takes a shorter collision)
 };
 
 struct Item {
