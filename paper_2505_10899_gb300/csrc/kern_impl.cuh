@@ -307,15 +307,15 @@ cudaError_t launch_lo_from_f64<LBM_T>(LBM_T* lo, const LBM_T* hi, const double* 
 template <>
 cudaError_t launch_volume_partial<LBM_T>(const CaseDev<LBM_T>* cases, const Item* items,
                                          int n_items, int bx, int parity, double* part,
-                                         cudaStream_t s) {
+                                         const VolumeEnd& end, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
   switch (bx) {
-    case 32: volume_partial<LBM_T, 32><<<n_items, 32, 0, s>>>(cases, items, parity, part); break;
-    case 64: volume_partial<LBM_T, 64><<<n_items, 64, 0, s>>>(cases, items, parity, part); break;
-    case 96: volume_partial<LBM_T, 96><<<n_items, 96, 0, s>>>(cases, items, parity, part); break;
-    case 128: volume_partial<LBM_T, 128><<<n_items, 128, 0, s>>>(cases, items, parity, part); break;
-    case 192: volume_partial<LBM_T, 192><<<n_items, 192, 0, s>>>(cases, items, parity, part); break;
-    case 256: volume_partial<LBM_T, 256><<<n_items, 256, 0, s>>>(cases, items, parity, part); break;
+    case 32: volume_partial<LBM_T, 32><<<n_items, 32, 0, s>>>(cases, items, parity, part, end); break;
+    case 64: volume_partial<LBM_T, 64><<<n_items, 64, 0, s>>>(cases, items, parity, part, end); break;
+    case 96: volume_partial<LBM_T, 96><<<n_items, 96, 0, s>>>(cases, items, parity, part, end); break;
+    case 128: volume_partial<LBM_T, 128><<<n_items, 128, 0, s>>>(cases, items, parity, part, end); break;
+    case 192: volume_partial<LBM_T, 192><<<n_items, 192, 0, s>>>(cases, items, parity, part, end); break;
+    case 256: volume_partial<LBM_T, 256><<<n_items, 256, 0, s>>>(cases, items, parity, part, end); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

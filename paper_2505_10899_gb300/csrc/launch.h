@@ -104,10 +104,12 @@ cudaError_t launch_add_lo_f64(double* v, const T* lo, int64_t n, cudaStream_t s)
 template <typename T>
 cudaError_t launch_lo_from_f64(T* lo, const T* hi, const double* v, int64_t n, cudaStream_t s);
 
-// Per-item partial volumes (labelled regions) of the state in buffer parity.
+// Per-item partial volumes (labelled regions) of the state in buffer parity;
+// with end.ticket also the per-case sums, by the CTA that finishes last.
 template <typename T>
 cudaError_t launch_volume_partial(const CaseDev<T>* cases, const Item* items, int n_items,
-                                  int bx, int parity, double* part, cudaStream_t s);
+                                  int bx, int parity, double* part, const VolumeEnd& end,
+                                  cudaStream_t s);
 
 // Per-case sums of the item partials (written by the step kernel's fused
 // volume or by launch_volume_partial): the cases case_ids[0..ncases), or

@@ -277,7 +277,8 @@ Layout make_layout(const lbm_params* c, int n, int n_items, int total_regions,
   L.part = off;
   off = align_up(off + (size_t)n_items * lbmk::kMaxRegions * sizeof(double));
   L.vol = off;
-  off = align_up(off + (size_t)std::max(total_regions, n * lbmk::kMaxRegions) * sizeof(double));
+  // volumes, and a copy of the error flags behind them
+  off = align_up(off + (size_t)(std::max(total_regions, n * lbmk::kMaxRegions) + 1) * sizeof(double));
   L.init = off;
   off = align_up(off + (size_t)n * sizeof(lbmk::InitSrc));
   L.chainc = off;  // case indices, chain by chain
@@ -665,14 +666,61 @@ int check_case(const lbm_handle* h, int c) {
   return LBM_OK;
 }
 
-int read_flags(lbm_handle* h) {
-  int32_t fl = 0;
-  LBM_CUDA(cudaMemcpyAsync(&fl, h->flags, sizeof fl, cudaMemcpyDeviceToHost, h->stream));
-  LBM_CUDA(cudaStreamSynchronize(h->stream));
+int flags_status(int32_t fl) {
   if (fl & lbmk::kFlagBounds)
     return fail(LBM_ERR_BOUNDS, "index out of range (build with index checks)");
   if (fl & lbmk::kFlagTimeout) return fail(LBM_ERR_TIMEOUT, "a bounded device wait timed out");
   if (fl & lbmk::kFlagNonFinite) return fail(LBM_ERR_NONFINITE, "non-finite macroscopic field");
+  return LBM_OK;
+}
+
+int read_flags(lbm_handle* h) {
+  int32_t fl = 0;
+  LBM_CUDA(cudaMemcpyAsync(&fl, h->flags, sizeof fl, cudaMemcpyDeviceToHost, h->stream));
+  LBM_CUDA(cudaStreamSynchronize(h->stream));
+  return flags_status(fl);
+}
+
+// Volumes of every case into `out` (device).  flags_out: where the one-launch
+// form leaves a copy of the error flags; *fused says whether it ran.  One
+// launch where one chain holds few items: above a few hundred the last CTA's
+// sums would outlast the second launch.
+constexpr int kVolumeFusedItems = 1024;
+constexpr int kVolumeFusedRegions = 64;
+
+int enqueue_volume(lbm_handle* h, double* out, int32_t* flags_out, bool* fused) {
+  cudaError_t e = cudaSuccess;
+  *fused = h->nchains == 1 && (int)h->items.size() <= kVolumeFusedItems &&
+           h->total_regions <= kVolumeFusedRegions;
+  lbmk::VolumeEnd end{};
+  if (*fused) {
+    end.ticket = (unsigned int*)(h->ws + h->L.hdr + 40);
+    end.ncases = h->ncases;
+    end.out = out;
+    end.flags = h->flags;
+    end.flags_out = flags_out;
+  }
+  // item partials chain by chain (each chain's strip width), then the cases
+  for (int c = 0; c < h->nchains && e == cudaSuccess; ++c) {
+    const int i0 = h->chain_item[c], ni = h->chain_item[c + 1] - i0;
+    double* part = h->part + (int64_t)i0 * lbmk::kMaxRegions;
+    if (h->precision == LBM_F32)
+      e = lbmk::launch_volume_partial<float>((const CaseDev<float>*)h->cases_dev, h->items_dev + i0,
+                                             ni, h->chain_bx[c], h->parity, part, end, h->stream);
+    else
+      e = lbmk::launch_volume_partial<double>((const CaseDev<double>*)h->cases_dev,
+                                              h->items_dev + i0, ni, h->chain_bx[c], h->parity,
+                                              part, end, h->stream);
+  }
+  if (e == cudaSuccess && !*fused) {
+    if (h->precision == LBM_F32)
+      e = lbmk::launch_volume_final<float>((const CaseDev<float>*)h->cases_dev, nullptr, h->ncases,
+                                           h->part, out, nullptr, 0, 0, 0, h->stream);
+    else
+      e = lbmk::launch_volume_final<double>((const CaseDev<double>*)h->cases_dev, nullptr,
+                                            h->ncases, h->part, out, nullptr, 0, 0, 0, h->stream);
+  }
+  if (e != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("volume: ") + cudaGetErrorString(e));
   return LBM_OK;
 }
 
@@ -1347,38 +1395,31 @@ int lbm_track_volume(lbm_handle* h, double* d_out) {
 int lbm_volume_async(lbm_handle* h, double* d_out) {
   lbmk::TraceRange trace("lbm_volume");
   if (!h || !d_out) return fail(LBM_ERR_ARG, "null argument");
-  cudaError_t e = cudaSuccess;
-  // item partials chain by chain (each chain's strip width), then the cases
-  for (int c = 0; c < h->nchains && e == cudaSuccess; ++c) {
-    const int i0 = h->chain_item[c], ni = h->chain_item[c + 1] - i0;
-    double* part = h->part + (int64_t)i0 * lbmk::kMaxRegions;
-    if (h->precision == LBM_F32)
-      e = lbmk::launch_volume_partial<float>((const CaseDev<float>*)h->cases_dev, h->items_dev + i0,
-                                             ni, h->chain_bx[c], h->parity, part, h->stream);
-    else
-      e = lbmk::launch_volume_partial<double>((const CaseDev<double>*)h->cases_dev,
-                                              h->items_dev + i0, ni, h->chain_bx[c], h->parity,
-                                              part, h->stream);
-  }
-  if (e == cudaSuccess) {
-    if (h->precision == LBM_F32)
-      e = lbmk::launch_volume_final<float>((const CaseDev<float>*)h->cases_dev, nullptr, h->ncases,
-                                           h->part, d_out, nullptr, 0, 0, 0, h->stream);
-    else
-      e = lbmk::launch_volume_final<double>((const CaseDev<double>*)h->cases_dev, nullptr,
-                                            h->ncases, h->part, d_out, nullptr, 0, 0, 0, h->stream);
-  }
-  if (e != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("volume: ") + cudaGetErrorString(e));
-  return LBM_OK;
+  bool fused;
+  return enqueue_volume(h, d_out, nullptr, &fused);
 }
 
 int lbm_volume(lbm_handle* h, double* h_out) {
+  lbmk::TraceRange trace("lbm_volume");
   if (!h || !h_out) return fail(LBM_ERR_ARG, "null argument");
-  int rc = lbm_volume_async(h, h->vol);
+  const size_t nv = (size_t)h->total_regions;
+  bool fused;
+  int rc = enqueue_volume(h, h->vol, (int32_t*)(h->vol + nv), &fused);
   if (rc) return rc;
-  LBM_CUDA(cudaMemcpyAsync(h_out, h->vol, h->total_regions * sizeof(double), cudaMemcpyDeviceToHost,
+  if (!fused) {
+    LBM_CUDA(cudaMemcpyAsync(h_out, h->vol, nv * sizeof(double), cudaMemcpyDeviceToHost,
+                             h->stream));
+    return read_flags(h);
+  }
+  // the volumes and the flags in one copy
+  double got[kVolumeFusedRegions + 1];
+  LBM_CUDA(cudaMemcpyAsync(got, h->vol, (nv + 1) * sizeof(double), cudaMemcpyDeviceToHost,
                            h->stream));
-  return read_flags(h);
+  LBM_CUDA(cudaStreamSynchronize(h->stream));
+  std::copy(got, got + nv, h_out);
+  int32_t fl;
+  memcpy(&fl, &got[nv], sizeof fl);
+  return flags_status(fl);
 }
 
 int lbm_fields(lbm_handle* h, int32_t c, double* phi, double* ux, double* uy, double* p) {

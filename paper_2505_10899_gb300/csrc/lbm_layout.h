@@ -108,6 +108,17 @@ struct ResRun {
   int64_t rec_stride;  // elements between recorded states
 };
 
+// End of a one-launch volume reduction (volume_partial): ticket word (0
+// between launches; null: partials only), cases, output, and a copy of the
+// error flags beside the volumes (flags_out may be null).
+struct VolumeEnd {
+  unsigned int* ticket;
+  int32_t ncases;
+  double* out;
+  const int32_t* flags;
+  int32_t* flags_out;
+};
+
 enum { kModeStep = 0, kModeFields = 1 };
 enum { kFlagNonFinite = 1, kFlagTimeout = 2 };
 
