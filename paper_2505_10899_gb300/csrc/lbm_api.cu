@@ -214,11 +214,11 @@ Plan make_plan(const lbm_params* c, int n, const Tiling& t, int nreq, bool rowmo
 // 8 cases run 19.1 us per step in 128 x 4, 21.6 in 64 x 4, 24.3 in 32 x 4).
 // Rows: a CTA of `rows` rows takes about rows + 2.5 row times in FP32 (the
 // halo rows and the prologue), and the step as many of these as it has waves
-// of resident CTAs: whole waves where one grid fills few of them, half a wave
-// of tail where there are many, or uneven cases and two chains.  Measured, us
-// per step (16 rows as the fixed choice -> this one): 1024^2 45.4 -> 42.8,
-// 2048^2 149 -> 134, 8192 x 4096 973 -> 964, 16 uneven cases 46.1 -> 39.0,
-// 512 cases 1173 -> 1144.  FP64 is bound by its pipe, which CTAs of one SM
+// of resident CTAs; the two chains of a batch run side by side, so their
+// waves overlap and each may fill the chip.  Measured, us per step (16 rows,
+// or narrow strips in small batches, -> this choice): 1024^2 45.4 -> 42.8,
+// 2048^2 149 -> 134, 8192 x 4096 973 -> 964; uneven cases: 12 27.0 -> 23.3, 16
+// 46.1 -> 39.0, 20 67.1 -> 62.4, 512 1173 -> 1138.  FP64 is bound by its pipe, which CTAs of one SM
 // share: the fullest SM decides, a halo row costs its phi and psi only, and
 // fewer than three CTAs per SM leave the pipe idle (2048^2 3045 -> 2967; 8
 // uneven cases of 237,000 nodes: 520 CTAs 209, 260 CTAs 236, 130 CTAs 272).
@@ -235,8 +235,9 @@ Tiling choose_tiling(const lbm_params* c, int n, bool tma) {
       break;
     }
   }
-  // CTAs of 128 threads per SM that the registers allow
-  const int slots = 152 * (128 / t.bx) * (tma ? 6 : 3);
+  // resident CTAs (6 or 3 of 128 threads per SM by their registers), for each
+  // of the default chains
+  const int64_t slots = (int64_t)152 * (128 / t.bx) * (tma ? 6 : 3) * std::min(2, n);
   double best = 1e300;
   for (int rows : {2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64}) {
     int64_t items = 0;
@@ -246,8 +247,7 @@ Tiling choose_tiling(const lbm_params* c, int n, bool tma) {
     if (c[0].precision == LBM_F64) {
       cost = (double)std::max<int64_t>((items + 151) / 152, 3) * (rows + 0.6);
     } else {
-      const double waves = (double)items / slots;
-      cost = (n == 1 && waves <= 4 ? std::ceil(waves) : std::max(1.0, waves + 0.5)) * (rows + 2.5);
+      cost = (double)((items + slots - 1) / slots) * (rows + 2.5);
     }
     if (cost < best) best = cost, t.rows = rows;
   }
