@@ -389,7 +389,11 @@ int lbm_adjoint_init(lbm_handle* h, const double* d_phi0, const double* d_u0,
  * t0 <= t < t0+count, is read from d_states + (t - t0) * stride_bytes
  * (snapshot layout, as lbm_record_steps writes it).  The count adjoint
  * steps (lbm_adjoint_step_from each) are enqueued in one call, alternating
- * between d_adj and d_spare (a second adjoint state); parameter derivatives
+ * between d_adj and d_spare (a second adjoint state), or, in FP32 on coupled
+ * grids that fit the SMs' shared memory (about 140,000 nodes) and outside
+ * stream capture, run in one cooperative launch (equal up to rounding; its
+ * waits are bounded as lbm_set_wait_limit says, and one that gives up raises
+ * LBM_ERR_TIMEOUT); parameter derivatives
  * accumulate on the device.  Asynchronous.  Errors: LBM_ERR_ARG,
  * LBM_ERR_WORKSPACE, LBM_ERR_CUDA. */
 int lbm_adjoint_sweep(lbm_handle* h, const void* d_states, int64_t stride_bytes, int64_t t0,

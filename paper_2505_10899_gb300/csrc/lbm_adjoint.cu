@@ -31,6 +31,8 @@
 
 #include "lbm_handle.h"
 #include "lbm_node.cuh"
+#include "lbm_res_plan.h"
+#include "lbm_resident.cuh"
 
 namespace lbmk {
 int set_last_error(int code, const char* msg);
@@ -212,16 +214,288 @@ __device__ __forceinline__ void ad_block_partials(double (&red)[kAdThreads / 32]
   }
 }
 
+// What one node's reverse step gives: the adjoints of its pulled inputs, of
+// phi*u of the previous step, of its own phi, and of the stencil differences.
+template <typename R>
+struct AdOut {
+  R lF[9], lG[9], ljpx, ljpy, lphi, lgpx, lgpy, llap, lqx, lqy;
+};
+
+// The reverse arithmetic of one node.  F, G: pulled populations (F with the
+// moving-wall term); Pv, Qv: phi and psi at the node and its neighbours; aF,
+// aG, aJx, aJy: adjoints of what the node stores; gacc: parameter terms.
+template <typename R>
+__device__ __forceinline__ AdOut<R> ad_node_math(const AdArgs<R>& a, int x, int y, const R (&F)[9],
+                                                 const R (&G)[9], R jpx, R jpy, const R (&Pv)[9],
+                                                 const R (&Qv)[9], const R (&aF)[9],
+                                                 const R (&aG)[9], R aJx, R aJy, bool wbot,
+                                                 bool wtop, R (&gacc)[kNParam]) {
+  using N = lbmk::Num<R>;
+  const int nx = a.nx, ny = a.ny;
+  const Phys<R>& ph = a.ph;
+  // ---------------- forward recompute (as node_update) ----------------
+  const R phi = Pv[0];
+  const R gpx = R(1.0 / 3.0) * (Pv[1] - Pv[3]) + R(1.0 / 12.0) * ((Pv[5] - Pv[6]) + (Pv[8] - Pv[7]));
+  const R gpy = R(1.0 / 3.0) * (Pv[2] - Pv[4]) + R(1.0 / 12.0) * ((Pv[5] - Pv[8]) + (Pv[6] - Pv[7]));
+  const R lap = R(2.0 / 3.0) * (((Pv[1] + Pv[3]) + (Pv[2] + Pv[4])) - R(4) * phi) +
+                R(1.0 / 6.0) * (((Pv[5] + Pv[6]) + (Pv[8] + Pv[7])) - R(4) * phi);
+  const R qx = R(4) * (Qv[1] - Qv[3]) + ((Qv[5] - Qv[6]) + (Qv[8] - Qv[7]));
+  const R qy = R(4) * (Qv[2] - Qv[4]) + ((Qv[5] - Qv[8]) + (Qv[6] - Qv[7]));
+  const R poly = phi * (phi - R(1)) * (phi - R(0.5));
+  const R mu = ph.beta4 * poly - ph.kappa * lap;
+  const R Fx = mu * gpx, Fy = mu * gpy;
+  R ux, uy;
+  R rho = R(1), irho = R(1), Rx = R(0), Ry = R(0), u2 = R(0), mu_v = R(0), s7 = a.s7;
+  R sD7 = a.sD7, hD7 = a.hD7;
+  Mom<R> mf{};
+  if (a.coupled) {
+    rho = a.rho_g + phi * a.drho;
+    irho = N::rcp(rho);  // the reciprocal the forward step takes
+    mf = lbmk::moments(F);
+    ux = (mf.m3 + R(0.5) * Fx) * irho;
+    uy = (mf.m5 + R(0.5) * Fy) * irho;
+    Rx = a.drho * gpx;
+    Ry = a.drho * gpy;
+    u2 = ux * ux + uy * uy;
+    if (a.var_tau) {
+      mu_v = a.mu_g + phi * a.dmu;
+      const R tau = R(3) * mu_v * irho + R(0.5);
+      s7 = N::rcp(tau);
+      sD7 = R(-0.25) * s7;
+      hD7 = R(0.25) - R(0.125) * s7;
+    }
+  } else {
+    R sx, cx, sy, cy;
+    N::sincospi_((R(x) + R(0.5)) / R(nx), &sx, &cx);
+    N::sincospi_((R(y) + R(0.5)) / R(ny), &sy, &cy);
+    ux = -a.ct * (sx * sx) * (R(2) * sy * cy);
+    uy = a.ct * (sy * sy) * (R(2) * sx * cx);
+  }
+  const R Jx = phi * ux, Jy = phi * uy;
+  const R dJx = Jx - jpx, dJy = Jy - jpy;
+  const R pc = N::clamp01(phi);
+  const R ta = pc + ph.xi, tb = (R(1) - pc) + ph.xi;
+  const R q2 = qx * qx + qy * qy;
+  const R iq = (q2 >= ph.qmin2) ? N::rsq(q2) : R(0);
+  const R sh = ph.lamW * ph.tfac * ta * tb * iq;
+  const R Vx = R(3) * dJx + sh * qx, Vy = R(3) * dJy + sh * qy;
+  const Mom<R> mg = lbmk::moments(G);
+
+  // ---------------- reverse ----------------
+  R lphi = R(0), lmu = R(0), lgpx = R(0), lgpy = R(0), llap = R(0), lqx = R(0), lqy = R(0);
+  R lux = R(0), luy = R(0);
+  // g*_0 = phi - sum_{i>=1} g*'_i; g*' = G + M^T e (e0 = 0)
+  lphi += aG[0];
+  R aGp[9];
+  aGp[0] = R(0);
+  #pragma unroll
+  for (int i = 1; i < 9; ++i) aGp[i] = aG[i] - aG[0];
+  R lG[9];
+  #pragma unroll
+  for (int i = 0; i < 9; ++i) lG[i] = aGp[i];
+  const Mom<R> le = lbmk::moments(aGp);  // lambda_e = M lambda_g*'
+  R lmg[9] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
+  R lLam = R(0), lJx = R(0), lJy = R(0), lVx = R(0), lVy = R(0);
+  // e1, e2
+  lmg[1] += ph.gsD[1] * le.m1;
+  lLam += R(-2) * ph.gsD[1] * le.m1;
+  lphi += R(4) * ph.gsD[1] * le.m1;
+  lmg[2] += ph.gsD[2] * le.m2;
+  lphi += R(-4) * ph.gsD[2] * le.m2;
+  lLam += R(3) * ph.gsD[2] * le.m2;
+  // e3..e6
+  lmg[3] += ph.gsD[3] * le.m3;
+  lJx += -ph.gsD[3] * le.m3;
+  lVx += ph.ghD3[3] * le.m3;
+  lmg[4] += ph.gsD[4] * le.m4;
+  lJx += ph.gsD[4] * le.m4;
+  lVx += -ph.ghD3[4] * le.m4;
+  lmg[5] += ph.gsD[5] * le.m5;
+  lJy += -ph.gsD[5] * le.m5;
+  lVy += ph.ghD3[5] * le.m5;
+  lmg[6] += ph.gsD[6] * le.m6;
+  lJy += ph.gsD[6] * le.m6;
+  lVy += -ph.ghD3[6] * le.m6;
+  lmg[7] += ph.gsD[7] * le.m7;
+  lmg[8] += ph.gsD[8] * le.m8;
+  {  // tau_g: s3 = s5 = 1/tau_g; gsD = -s/6, ghD3 = (1 - s/2)/18
+    const R lgs = (mg.m3 - Jx) * le.m3 + (mg.m5 - Jy) * le.m5;
+    const R lgh = Vx * le.m3 + Vy * le.m5;
+    const R ls = -lgs * R(1.0 / 6.0) - lgh * R(1.0 / 36.0);
+    const R sg = R(-6) * ph.gsD[3];  // = 1/tau_g
+    gacc[3] += -sg * sg * ls;
+  }
+  // mg = M G
+  lbmk::add_back(lG, lmg[0], lmg[1], lmg[2], lmg[3], lmg[4], lmg[5], lmg[6], lmg[7], lmg[8]);
+  // Lam = mu + lambda phi
+  lmu += lLam;
+  lphi += ph.lambda * lLam;
+  gacc[2] += phi * lLam;
+  // V = 3 dJ + sh q
+  const R ldJx = R(3) * lVx, ldJy = R(3) * lVy;
+  const R lsh = qx * lVx + qy * lVy;
+  lqx += sh * lVx;
+  lqy += sh * lVy;
+  // sh = lamW tfac ta tb iq
+  const R c0 = ph.lamW * ph.tfac;
+  const R lta = c0 * tb * iq * lsh, ltb = c0 * ta * iq * lsh, liq = c0 * ta * tb * lsh;
+  gacc[2] += ph.tfac * ta * tb * iq * lsh * a.invW;  // lamW = lambda / W
+  if (q2 >= ph.qmin2) {  // below the threshold n = 0: no derivative
+    const R lq2 = R(-0.5) * iq * iq * iq * liq;
+    lqx += R(2) * qx * lq2;
+    lqy += R(2) * qy * lq2;
+  }
+  if (phi > R(0) && phi < R(1)) lphi += lta - ltb;
+  // dJ = J - J_prev; J also stored
+  lJx += ldJx + aJx;
+  lJy += ldJy + aJy;
+  const R ljpx = -ldJx, ljpy = -ldJy;
+  // J = phi u
+  lphi += ux * lJx + uy * lJy;
+  lux += phi * lJx;
+  luy += phi * lJy;
+
+  R lF[9];
+  #pragma unroll
+  for (int i = 0; i < 9; ++i) lF[i] = R(0);
+  if (a.coupled) {
+    #pragma unroll
+    for (int i = 0; i < 9; ++i) lF[i] = aF[i];
+    const Mom<R> ld = lbmk::moments(aF);  // lambda_d = M lambda_f*
+    R lm[9] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
+    R lp = R(0), lru2 = R(0), luR = R(0), ljx = R(0), ljy = R(0), lFx = R(0), lFy = R(0);
+    R lrho = R(0), lRx = R(0), lRy = R(0), lsD7 = R(0), lhD7 = R(0), lirho = R(0), lu2 = R(0);
+    const R jx = rho * ux;
+    // d0..d6
+    lm[0] += ph.fsD[0] * ld.m0;
+    luR += ph.fhD[0] * ld.m0;
+    lm[1] += ph.fsD[1] * ld.m1;
+    lp += R(-6) * ph.fsD[1] * ld.m1;
+    lru2 += R(-3) * ph.fsD[1] * ld.m1;
+    lm[2] += ph.fsD[2] * ld.m2;
+    lp += R(9) * ph.fsD[2] * ld.m2;
+    lru2 += R(3) * ph.fsD[2] * ld.m2;
+    luR += -ph.fhD[2] * ld.m2;
+    lm[3] += ph.fsD[3] * ld.m3;
+    ljx += -ph.fsD[3] * ld.m3;
+    lFx += ph.fhD[3] * ld.m3;
+    lm[4] += ph.fsD[4] * ld.m4;
+    ljx += ph.fsD[4] * ld.m4;
+    lFx += -ph.fhD[4] * ld.m4;
+    lm[5] += ph.fsD[5] * ld.m5;
+    ljy += -ph.fsD[5] * ld.m5;
+    lFy += ph.fhD[5] * ld.m5;
+    lm[6] += ph.fsD[6] * ld.m6;
+    ljy += ph.fsD[6] * ld.m6;
+    lFy += -ph.fhD[6] * ld.m6;
+    // d7 = sD7 (m7 - rho(ux^2 - uy^2)) + hD7 (2/3)(ux Rx - uy Ry)
+    lm[7] += sD7 * ld.m7;
+    lrho += -sD7 * (ux * ux - uy * uy) * ld.m7;
+    lux += R(-2) * sD7 * rho * ux * ld.m7 + hD7 * R(2.0 / 3.0) * Rx * ld.m7;
+    luy += R(2) * sD7 * rho * uy * ld.m7 - hD7 * R(2.0 / 3.0) * Ry * ld.m7;
+    lRx += hD7 * R(2.0 / 3.0) * ux * ld.m7;
+    lRy += -hD7 * R(2.0 / 3.0) * uy * ld.m7;
+    lsD7 += (mf.m7 - rho * (ux * ux - uy * uy)) * ld.m7;
+    lhD7 += R(2.0 / 3.0) * (ux * Rx - uy * Ry) * ld.m7;
+    // d8 = sD7 (m8 - jx uy) + hD7 (1/3)(ux Ry + uy Rx)
+    lm[8] += sD7 * ld.m8;
+    ljx += -sD7 * uy * ld.m8;
+    luy += -sD7 * jx * ld.m8 + hD7 * R(1.0 / 3.0) * Rx * ld.m8;
+    lux += hD7 * R(1.0 / 3.0) * Ry * ld.m8;
+    lRy += hD7 * R(1.0 / 3.0) * ux * ld.m8;
+    lRx += hD7 * R(1.0 / 3.0) * uy * ld.m8;
+    lsD7 += (mf.m8 - jx * uy) * ld.m8;
+    lhD7 += R(1.0 / 3.0) * (ux * Ry + uy * Rx) * ld.m8;
+    // s7 (= s8): sD7 = -s7/4, hD7 = 1/4 - s7/8
+    const R ls7 = R(-0.25) * lsD7 - R(0.125) * lhD7;
+    if (a.var_tau) {
+      const R ltau = -s7 * s7 * ls7;  // s7 = 1/tau
+      const R lmuv = R(3) * irho * ltau;
+      lirho += R(3) * mu_v * ltau;
+      lphi += a.dmu * lmuv;
+    } else {
+      gacc[4] += -s7 * s7 * ls7;  // s7 = 1/tau_f
+    }
+    // jx = rho ux, jy = rho uy
+    lrho += ux * ljx + uy * ljy;
+    lux += rho * ljx;
+    luy += rho * ljy;
+    // ru2 = rho u2
+    lrho += u2 * lru2;
+    lu2 += rho * lru2;
+    // p = 0.6((m0 - F0) + uR/2 - (2/3) rho u2)
+    lm[0] += R(0.6) * lp;
+    lF[0] += R(-0.6) * lp;
+    luR += R(0.3) * lp;
+    lrho += R(-0.4) * u2 * lp;
+    lu2 += R(-0.4) * rho * lp;
+    // u2, uR
+    lux += R(2) * ux * lu2 + Rx * luR;
+    luy += R(2) * uy * lu2 + Ry * luR;
+    lRx += ux * luR;
+    lRy += uy * luR;
+    // R = drho grad phi
+    lgpx += a.drho * lRx;
+    lgpy += a.drho * lRy;
+    // u = (m + F/2) irho
+    lm[3] += irho * lux;
+    lFx += R(0.5) * irho * lux;
+    lirho += (mf.m3 + R(0.5) * Fx) * lux;
+    lm[5] += irho * luy;
+    lFy += R(0.5) * irho * luy;
+    lirho += (mf.m5 + R(0.5) * Fy) * luy;
+    // m = M F
+    lbmk::add_back(lF, lm[0], lm[1], lm[2], lm[3], lm[4], lm[5], lm[6], lm[7], lm[8]);
+    // moving-wall term: F_i += rho c_ix u_w / 6, rho = rho_g + phi drho
+    if (wbot) {
+      const R l = (lF[5] - lF[6]) * R(1.0 / 6.0);
+      lrho += a.u_bot * l;
+      gacc[6] += rho * l;
+    }
+    if (wtop) {
+      const R l = (lF[8] - lF[7]) * R(1.0 / 6.0);
+      lrho += a.u_top * l;
+      gacc[5] += rho * l;
+    }
+    // irho = 1/rho, rho = rho_g + phi drho
+    lrho += -irho * irho * lirho;
+    lphi += a.drho * lrho;
+    // F = mu grad phi
+    lmu += gpx * lFx + gpy * lFy;
+    lgpx += mu * lFx;
+    lgpy += mu * lFy;
+  }
+  // mu = beta4 poly - kappa lap
+  lphi += ph.beta4 * (R(3) * phi * phi - R(3) * phi + R(0.5)) * lmu;
+  llap += -ph.kappa * lmu;
+  gacc[0] += poly * lmu;
+  gacc[1] += -lap * lmu;
+
+  AdOut<R> o;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    o.lF[i] = lF[i];
+    o.lG[i] = lG[i];
+  }
+  o.ljpx = ljpx;
+  o.ljpy = ljpy;
+  o.lphi = lphi;
+  o.lgpx = lgpx;
+  o.lgpy = lgpy;
+  o.llap = llap;
+  o.lqx = lqx;
+  o.lqy = lqy;
+  return o;
+}
+
 // The per-node reverse sweep.  R is the arithmetic and storage type of the
 // states and adjoints (the handle's precision); the parameter partials are
 // summed per thread and per warp in R and accumulated in FP64 above that.
 template <typename R>
 __global__ void __launch_bounds__(kAdThreads, sizeof(R) == 4 ? 3 : 1) ad_node(const AdArgs<R> a) {
   __shared__ double red[kAdThreads / 32][kNParam];
-  using N = lbmk::Num<R>;
   const int nx = a.nx, ny = a.ny;
   const int64_t n = (int64_t)nx * ny, P = a.P;
-  const Phys<R>& ph = a.ph;
   // Parameter terms: each thread sums its nodes' terms and each warp its
   // threads' sums in R; the warp sums enter the FP64 block and CTA partials.
   // Under FP32 a 32-term FP32 partial adds rounding of the order of the
@@ -263,55 +537,6 @@ __global__ void __launch_bounds__(kAdThreads, sizeof(R) == 4 ? 3 : 1) ad_node(co
         F[8] += d;
       }
     }
-    // ---------------- forward recompute (as node_update) ----------------
-    const R phi = Pv[0];
-    const R gpx = R(1.0 / 3.0) * (Pv[1] - Pv[3]) + R(1.0 / 12.0) * ((Pv[5] - Pv[6]) + (Pv[8] - Pv[7]));
-    const R gpy = R(1.0 / 3.0) * (Pv[2] - Pv[4]) + R(1.0 / 12.0) * ((Pv[5] - Pv[8]) + (Pv[6] - Pv[7]));
-    const R lap = R(2.0 / 3.0) * (((Pv[1] + Pv[3]) + (Pv[2] + Pv[4])) - R(4) * phi) +
-                  R(1.0 / 6.0) * (((Pv[5] + Pv[6]) + (Pv[8] + Pv[7])) - R(4) * phi);
-    const R qx = R(4) * (Qv[1] - Qv[3]) + ((Qv[5] - Qv[6]) + (Qv[8] - Qv[7]));
-    const R qy = R(4) * (Qv[2] - Qv[4]) + ((Qv[5] - Qv[8]) + (Qv[6] - Qv[7]));
-    const R poly = phi * (phi - R(1)) * (phi - R(0.5));
-    const R mu = ph.beta4 * poly - ph.kappa * lap;
-    const R Fx = mu * gpx, Fy = mu * gpy;
-    R ux, uy;
-    R rho = R(1), irho = R(1), Rx = R(0), Ry = R(0), u2 = R(0), mu_v = R(0), s7 = a.s7;
-    R sD7 = a.sD7, hD7 = a.hD7;
-    Mom<R> mf{};
-    if (a.coupled) {
-      rho = a.rho_g + phi * a.drho;
-      irho = N::rcp(rho);  // the reciprocal the forward step takes
-      mf = lbmk::moments(F);
-      ux = (mf.m3 + R(0.5) * Fx) * irho;
-      uy = (mf.m5 + R(0.5) * Fy) * irho;
-      Rx = a.drho * gpx;
-      Ry = a.drho * gpy;
-      u2 = ux * ux + uy * uy;
-      if (a.var_tau) {
-        mu_v = a.mu_g + phi * a.dmu;
-        const R tau = R(3) * mu_v * irho + R(0.5);
-        s7 = N::rcp(tau);
-        sD7 = R(-0.25) * s7;
-        hD7 = R(0.25) - R(0.125) * s7;
-      }
-    } else {
-      R sx, cx, sy, cy;
-      N::sincospi_((R(x) + R(0.5)) / R(nx), &sx, &cx);
-      N::sincospi_((R(y) + R(0.5)) / R(ny), &sy, &cy);
-      ux = -a.ct * (sx * sx) * (R(2) * sy * cy);
-      uy = a.ct * (sy * sy) * (R(2) * sx * cx);
-    }
-    const R Jx = phi * ux, Jy = phi * uy;
-    const R dJx = Jx - jpx, dJy = Jy - jpy;
-    const R pc = N::clamp01(phi);
-    const R ta = pc + ph.xi, tb = (R(1) - pc) + ph.xi;
-    const R q2 = qx * qx + qy * qy;
-    const R iq = (q2 >= ph.qmin2) ? N::rsq(q2) : R(0);
-    const R sh = ph.lamW * ph.tfac * ta * tb * iq;
-    const R Vx = R(3) * dJx + sh * qx, Vy = R(3) * dJy + sh * qy;
-    const Mom<R> mg = lbmk::moments(G);
-
-    // ---------------- reverse ----------------
     R aF[9], aG[9];
     #pragma unroll
     for (int i = 0; i < 9; ++i) {
@@ -319,201 +544,15 @@ __global__ void __launch_bounds__(kAdThreads, sizeof(R) == 4 ? 3 : 1) ad_node(co
       aG[i] = a.ain[(9 + i) * n + k];
     }
     const R aJx = a.ain[18 * n + k], aJy = a.ain[19 * n + k];
-
-    R lphi = R(0), lmu = R(0), lgpx = R(0), lgpy = R(0), llap = R(0), lqx = R(0), lqy = R(0);
-    R lux = R(0), luy = R(0);
-    // g*_0 = phi - sum_{i>=1} g*'_i; g*' = G + M^T e (e0 = 0)
-    lphi += aG[0];
-    R aGp[9];
-    aGp[0] = R(0);
-    #pragma unroll
-    for (int i = 1; i < 9; ++i) aGp[i] = aG[i] - aG[0];
-    R lG[9];
-    #pragma unroll
-    for (int i = 0; i < 9; ++i) lG[i] = aGp[i];
-    const Mom<R> le = lbmk::moments(aGp);  // lambda_e = M lambda_g*'
-    R lmg[9] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
-    R lLam = R(0), lJx = R(0), lJy = R(0), lVx = R(0), lVy = R(0);
-    // e1, e2
-    lmg[1] += ph.gsD[1] * le.m1;
-    lLam += R(-2) * ph.gsD[1] * le.m1;
-    lphi += R(4) * ph.gsD[1] * le.m1;
-    lmg[2] += ph.gsD[2] * le.m2;
-    lphi += R(-4) * ph.gsD[2] * le.m2;
-    lLam += R(3) * ph.gsD[2] * le.m2;
-    // e3..e6
-    lmg[3] += ph.gsD[3] * le.m3;
-    lJx += -ph.gsD[3] * le.m3;
-    lVx += ph.ghD3[3] * le.m3;
-    lmg[4] += ph.gsD[4] * le.m4;
-    lJx += ph.gsD[4] * le.m4;
-    lVx += -ph.ghD3[4] * le.m4;
-    lmg[5] += ph.gsD[5] * le.m5;
-    lJy += -ph.gsD[5] * le.m5;
-    lVy += ph.ghD3[5] * le.m5;
-    lmg[6] += ph.gsD[6] * le.m6;
-    lJy += ph.gsD[6] * le.m6;
-    lVy += -ph.ghD3[6] * le.m6;
-    lmg[7] += ph.gsD[7] * le.m7;
-    lmg[8] += ph.gsD[8] * le.m8;
-    {  // tau_g: s3 = s5 = 1/tau_g; gsD = -s/6, ghD3 = (1 - s/2)/18
-      const R lgs = (mg.m3 - Jx) * le.m3 + (mg.m5 - Jy) * le.m5;
-      const R lgh = Vx * le.m3 + Vy * le.m5;
-      const R ls = -lgs * R(1.0 / 6.0) - lgh * R(1.0 / 36.0);
-      const R sg = R(-6) * ph.gsD[3];  // = 1/tau_g
-      gacc[3] += -sg * sg * ls;
-    }
-    // mg = M G
-    lbmk::add_back(lG, lmg[0], lmg[1], lmg[2], lmg[3], lmg[4], lmg[5], lmg[6], lmg[7], lmg[8]);
-    // Lam = mu + lambda phi
-    lmu += lLam;
-    lphi += ph.lambda * lLam;
-    gacc[2] += phi * lLam;
-    // V = 3 dJ + sh q
-    const R ldJx = R(3) * lVx, ldJy = R(3) * lVy;
-    const R lsh = qx * lVx + qy * lVy;
-    lqx += sh * lVx;
-    lqy += sh * lVy;
-    // sh = lamW tfac ta tb iq
-    const R c0 = ph.lamW * ph.tfac;
-    const R lta = c0 * tb * iq * lsh, ltb = c0 * ta * iq * lsh, liq = c0 * ta * tb * lsh;
-    gacc[2] += ph.tfac * ta * tb * iq * lsh * a.invW;  // lamW = lambda / W
-    if (q2 >= ph.qmin2) {  // below the threshold n = 0: no derivative
-      const R lq2 = R(-0.5) * iq * iq * iq * liq;
-      lqx += R(2) * qx * lq2;
-      lqy += R(2) * qy * lq2;
-    }
-    if (phi > R(0) && phi < R(1)) lphi += lta - ltb;
-    // dJ = J - J_prev; J also stored
-    lJx += ldJx + aJx;
-    lJy += ldJy + aJy;
-    const R ljpx = -ldJx, ljpy = -ldJy;
-    // J = phi u
-    lphi += ux * lJx + uy * lJy;
-    lux += phi * lJx;
-    luy += phi * lJy;
-
-    R lF[9];
-    #pragma unroll
-    for (int i = 0; i < 9; ++i) lF[i] = R(0);
-    if (a.coupled) {
-      #pragma unroll
-      for (int i = 0; i < 9; ++i) lF[i] = aF[i];
-      const Mom<R> ld = lbmk::moments(aF);  // lambda_d = M lambda_f*
-      R lm[9] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
-      R lp = R(0), lru2 = R(0), luR = R(0), ljx = R(0), ljy = R(0), lFx = R(0), lFy = R(0);
-      R lrho = R(0), lRx = R(0), lRy = R(0), lsD7 = R(0), lhD7 = R(0), lirho = R(0), lu2 = R(0);
-      const R jx = rho * ux;
-      // d0..d6
-      lm[0] += ph.fsD[0] * ld.m0;
-      luR += ph.fhD[0] * ld.m0;
-      lm[1] += ph.fsD[1] * ld.m1;
-      lp += R(-6) * ph.fsD[1] * ld.m1;
-      lru2 += R(-3) * ph.fsD[1] * ld.m1;
-      lm[2] += ph.fsD[2] * ld.m2;
-      lp += R(9) * ph.fsD[2] * ld.m2;
-      lru2 += R(3) * ph.fsD[2] * ld.m2;
-      luR += -ph.fhD[2] * ld.m2;
-      lm[3] += ph.fsD[3] * ld.m3;
-      ljx += -ph.fsD[3] * ld.m3;
-      lFx += ph.fhD[3] * ld.m3;
-      lm[4] += ph.fsD[4] * ld.m4;
-      ljx += ph.fsD[4] * ld.m4;
-      lFx += -ph.fhD[4] * ld.m4;
-      lm[5] += ph.fsD[5] * ld.m5;
-      ljy += -ph.fsD[5] * ld.m5;
-      lFy += ph.fhD[5] * ld.m5;
-      lm[6] += ph.fsD[6] * ld.m6;
-      ljy += ph.fsD[6] * ld.m6;
-      lFy += -ph.fhD[6] * ld.m6;
-      // d7 = sD7 (m7 - rho(ux^2 - uy^2)) + hD7 (2/3)(ux Rx - uy Ry)
-      lm[7] += sD7 * ld.m7;
-      lrho += -sD7 * (ux * ux - uy * uy) * ld.m7;
-      lux += R(-2) * sD7 * rho * ux * ld.m7 + hD7 * R(2.0 / 3.0) * Rx * ld.m7;
-      luy += R(2) * sD7 * rho * uy * ld.m7 - hD7 * R(2.0 / 3.0) * Ry * ld.m7;
-      lRx += hD7 * R(2.0 / 3.0) * ux * ld.m7;
-      lRy += -hD7 * R(2.0 / 3.0) * uy * ld.m7;
-      lsD7 += (mf.m7 - rho * (ux * ux - uy * uy)) * ld.m7;
-      lhD7 += R(2.0 / 3.0) * (ux * Rx - uy * Ry) * ld.m7;
-      // d8 = sD7 (m8 - jx uy) + hD7 (1/3)(ux Ry + uy Rx)
-      lm[8] += sD7 * ld.m8;
-      ljx += -sD7 * uy * ld.m8;
-      luy += -sD7 * jx * ld.m8 + hD7 * R(1.0 / 3.0) * Rx * ld.m8;
-      lux += hD7 * R(1.0 / 3.0) * Ry * ld.m8;
-      lRy += hD7 * R(1.0 / 3.0) * ux * ld.m8;
-      lRx += hD7 * R(1.0 / 3.0) * uy * ld.m8;
-      lsD7 += (mf.m8 - jx * uy) * ld.m8;
-      lhD7 += R(1.0 / 3.0) * (ux * Ry + uy * Rx) * ld.m8;
-      // s7 (= s8): sD7 = -s7/4, hD7 = 1/4 - s7/8
-      const R ls7 = R(-0.25) * lsD7 - R(0.125) * lhD7;
-      if (a.var_tau) {
-        const R ltau = -s7 * s7 * ls7;  // s7 = 1/tau
-        const R lmuv = R(3) * irho * ltau;
-        lirho += R(3) * mu_v * ltau;
-        lphi += a.dmu * lmuv;
-      } else {
-        gacc[4] += -s7 * s7 * ls7;  // s7 = 1/tau_f
-      }
-      // jx = rho ux, jy = rho uy
-      lrho += ux * ljx + uy * ljy;
-      lux += rho * ljx;
-      luy += rho * ljy;
-      // ru2 = rho u2
-      lrho += u2 * lru2;
-      lu2 += rho * lru2;
-      // p = 0.6((m0 - F0) + uR/2 - (2/3) rho u2)
-      lm[0] += R(0.6) * lp;
-      lF[0] += R(-0.6) * lp;
-      luR += R(0.3) * lp;
-      lrho += R(-0.4) * u2 * lp;
-      lu2 += R(-0.4) * rho * lp;
-      // u2, uR
-      lux += R(2) * ux * lu2 + Rx * luR;
-      luy += R(2) * uy * lu2 + Ry * luR;
-      lRx += ux * luR;
-      lRy += uy * luR;
-      // R = drho grad phi
-      lgpx += a.drho * lRx;
-      lgpy += a.drho * lRy;
-      // u = (m + F/2) irho
-      lm[3] += irho * lux;
-      lFx += R(0.5) * irho * lux;
-      lirho += (mf.m3 + R(0.5) * Fx) * lux;
-      lm[5] += irho * luy;
-      lFy += R(0.5) * irho * luy;
-      lirho += (mf.m5 + R(0.5) * Fy) * luy;
-      // m = M F
-      lbmk::add_back(lF, lm[0], lm[1], lm[2], lm[3], lm[4], lm[5], lm[6], lm[7], lm[8]);
-      // moving-wall term: F_i += rho c_ix u_w / 6, rho = rho_g + phi drho
-      if (wbot) {
-        const R l = (lF[5] - lF[6]) * R(1.0 / 6.0);
-        lrho += a.u_bot * l;
-        gacc[6] += rho * l;
-      }
-      if (wtop) {
-        const R l = (lF[8] - lF[7]) * R(1.0 / 6.0);
-        lrho += a.u_top * l;
-        gacc[5] += rho * l;
-      }
-      // irho = 1/rho, rho = rho_g + phi drho
-      lrho += -irho * irho * lirho;
-      lphi += a.drho * lrho;
-      // F = mu grad phi
-      lmu += gpx * lFx + gpy * lFy;
-      lgpx += mu * lFx;
-      lgpy += mu * lFy;
-    }
-    // mu = beta4 poly - kappa lap
-    lphi += ph.beta4 * (R(3) * phi * phi - R(3) * phi + R(0.5)) * lmu;
-    llap += -ph.kappa * lmu;
-    gacc[0] += poly * lmu;
-    gacc[1] += -lap * lmu;
+    const AdOut<R> o =
+        ad_node_math(a, x, y, F, G, jpx, jpy, Pv, Qv, aF, aG, aJx, aJy, wbot, wtop, gacc);
+    const R lgpx = o.lgpx, lgpy = o.lgpy, llap = o.llap, lqx = o.lqx, lqy = o.lqy;
 
     // stencil adjoints (transpose of the difference forms above)
     const R gx3 = lgpx * R(1.0 / 3.0), gy3 = lgpy * R(1.0 / 3.0);
     const R gx12 = lgpx * R(1.0 / 12.0), gy12 = lgpy * R(1.0 / 12.0);
     const R la = R(2.0 / 3.0) * llap, ld6 = llap * R(1.0 / 6.0);
-    a.lP[0 * n + k] = R(-10.0 / 3.0) * llap + lphi;
+    a.lP[0 * n + k] = R(-10.0 / 3.0) * llap + o.lphi;
     a.lP[1 * n + k] = gx3 + la;
     a.lP[3 * n + k] = -gx3 + la;
     a.lP[2 * n + k] = gy3 + la;
@@ -535,11 +574,11 @@ __global__ void __launch_bounds__(kAdThreads, sizeof(R) == 4 ? 3 : 1) ad_node(co
     // walls included)
     #pragma unroll
     for (int i = 0; i < 9; ++i) {
-      a.aout[spl[i] * n + src[i]] = lF[i];
-      a.aout[(9 + spl[i]) * n + src[i]] = lG[i];
+      a.aout[spl[i] * n + src[i]] = o.lF[i];
+      a.aout[(9 + spl[i]) * n + src[i]] = o.lG[i];
     }
-    a.aout[18 * n + k] = ljpx;
-    a.aout[19 * n + k] = ljpy;
+    a.aout[18 * n + k] = o.ljpx;
+    a.aout[19 * n + k] = o.ljpy;
   }
   ad_block_partials(red, gacc, a.part);
 }
@@ -585,6 +624,8 @@ __global__ void __launch_bounds__(kAdThreads, 4) ad_gather(R* __restrict__ phi, 
     }
   }
 }
+
+#include "lbm_adjoint_resident.cuh"
 
 // Adjoint of the initial state map (local part): phi0 -> hbar0, g_eq, f_eq,
 // phi0 u0.  Writes the local phi0 adjoint and the adjoint of lap(phi0).
@@ -745,11 +786,27 @@ struct AdScratch {
   void *phi, *psi, *lP, *lQ;
   double *part, *sums;
   double *init_lphi, *init_llap;
+  lbmk::ResTile* tiles;  // chip-resident sweep: tiles, two sets of exchange slots
+  uint4* slots;
 };
 
 size_t elem_bytes(const lbm_handle* h) { return h->precision == LBM_F64 ? 8 : 4; }
 
 size_t planes_bytes(int64_t n, size_t es) { return (19 * (size_t)n * es + 255) / 256 * 256; }
+
+size_t base_bytes(int64_t n, size_t es) {
+  return planes_bytes(n, es) +
+         ((size_t)(kAdBlocks * kNParam + 8) * sizeof(double) + 255) / 256 * 256;
+}
+
+size_t tile_bytes(const lbmk::ResPlan& p) {
+  return (p.tiles.size() * sizeof(lbmk::ResTile) + 255) / 256 * 256;
+}
+
+size_t scratch_bytes(const lbm_handle* h, const lbmk::ResPlan& p) {
+  const int64_t n = (int64_t)h->params[0].nx * h->params[0].ny;
+  return base_bytes(n, elem_bytes(h)) + tile_bytes(p) + (size_t)2 * p.nslots * sizeof(uint4);
+}
 
 AdScratch carve(lbm_handle* h) {
   const int64_t n = (int64_t)h->params[0].nx * h->params[0].ny;
@@ -764,11 +821,10 @@ AdScratch carve(lbm_handle* h) {
   s.sums = s.part + kAdBlocks * kNParam;
   s.init_lphi = (double*)s.lP;  // 9 planes of es bytes hold 2 FP64 planes
   s.init_llap = s.init_lphi + n;
+  char* r = b + base_bytes(n, es);
+  s.tiles = (lbmk::ResTile*)r;
+  s.slots = (uint4*)(r + tile_bytes(h->adj_res));
   return s;
-}
-
-size_t scratch_bytes(int64_t n, size_t es) {
-  return planes_bytes(n, es) + (size_t)(kAdBlocks * kNParam + 8) * sizeof(double);
 }
 
 int check_handle(lbm_handle* h, bool need_ws) {
@@ -805,6 +861,20 @@ int take_grads(lbm_handle* h, double* out) {
   return LBM_OK;
 }
 
+// Whether the sweep kernel's CTAs are co-resident (and allow its memory).
+bool sweep_fits(int ntiles) {
+  int dev = 0, nsm = 0, per_sm = 0;
+  cudaError_t e = cudaFuncSetAttribute(ad_resident, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)AdShape::SMEM_BYTES);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ad_resident, kAdNT,
+                                                      AdShape::SMEM_BYTES);
+  if (e != cudaSuccess) cudaGetLastError();  // not available: the two-kernel sweep runs
+  return e == cudaSuccess && per_sm * nsm >= ntiles;
+}
+
 template <typename R>
 const CaseDev<R>& case0(const lbm_handle* h) {
   if constexpr (sizeof(R) == 4) return h->cf[0]; else return h->cd[0];
@@ -821,7 +891,7 @@ extern "C" {
 
 size_t lbm_adjoint_workspace_bytes(const lbm_handle* h) {
   if (!h || h->ncases != 1) return 0;
-  return scratch_bytes((int64_t)h->params[0].nx * h->params[0].ny, elem_bytes(h));
+  return scratch_bytes(h, lbmk::res_plan_adjoint(h->params[0]));
 }
 
 int lbm_adjoint_attach(lbm_handle* h, void* d_scratch, size_t bytes) {
@@ -832,8 +902,22 @@ int lbm_adjoint_attach(lbm_handle* h, void* d_scratch, size_t bytes) {
   if (bytes < lbm_adjoint_workspace_bytes(h)) return fail(LBM_ERR_WORKSPACE, "adjoint scratch too small");
   h->adj_ws = (char*)d_scratch;
   h->adj_ws_bytes = bytes;
-  cudaError_t e = cudaMemsetAsync(carve(h).part, 0, (kAdBlocks + 1) * kNParam * sizeof(double),
+  h->adj_res = lbmk::res_plan_adjoint(h->params[0]);
+  h->adj_epoch = 1;
+  const AdScratch s = carve(h);
+  cudaError_t e = cudaMemsetAsync(s.part, 0, (kAdBlocks + 1) * kNParam * sizeof(double),
                                   h->stream);  // partials and accumulator
+  if (e == cudaSuccess && h->adj_res.variant >= 0) {
+    if (!sweep_fits((int)h->adj_res.tiles.size())) {
+      h->adj_res.variant = -1;
+    } else {
+      e = cudaMemcpyAsync(s.tiles, h->adj_res.tiles.data(),
+                          h->adj_res.tiles.size() * sizeof(lbmk::ResTile), cudaMemcpyHostToDevice,
+                          h->stream);
+      if (e == cudaSuccess)
+        e = cudaMemsetAsync(s.slots, 0, (size_t)2 * h->adj_res.nslots * sizeof(uint4), h->stream);
+    }
+  }
   if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
   return LBM_OK;
 }
@@ -868,33 +952,17 @@ int lbm_adjoint_seed_phi(lbm_handle* h, const double* d_dphi, void* d_adj_state)
 
 namespace {
 
-// One adjoint step from the state S_t held in (fA, gA, JA) with plane stride
-// P at step index t (the handle's own buffers, or a snapshot).
-// phase_ready: phi and psi of S_t are already in the scratch planes (the
-// previous step of a sweep formed them); gB/PB: g planes of the state of the
-// next step of a sweep, whose phi and psi the gather launch forms, or null.
+// What every adjoint step of a handle shares, at step index t.
 template <typename R>
-int adjoint_step_impl(lbm_handle* h, const R* fA, const R* gA, const R* JA, int64_t P, int64_t t,
-                      const void* d_adj_in, void* d_adj_out, double* h_param_grads,
-                      bool phase_ready = false, const R* gB = nullptr, int64_t PB = 0) {
+AdArgs<R> ad_args(const lbm_handle* h, const AdScratch& s, int64_t t) {
   const lbm_params& p = h->params[0];
   const CaseDev<R>& cd = case0<R>(h);
   const bool coupled = h->flow == LBM_FLOW_COUPLED;
-  AdScratch s = carve(h);
-  if (!phase_ready)
-    ad_phase<R><<<kAdBlocks, kAdThreads, 0, h->stream>>>(gA, P, p.nx, p.ny, p.walls, (R)p.xi,
-                                                         (R*)s.phi, (R*)s.psi);
   AdArgs<R> a{};
-  a.fA = coupled ? fA : nullptr;
-  a.gA = gA;
-  a.JA = JA;
-  a.P = P;
   a.nx = p.nx;
   a.ny = p.ny;
   a.phi = (const R*)s.phi;
   a.psi = (const R*)s.psi;
-  a.ain = (const R*)d_adj_in;
-  a.aout = (R*)d_adj_out;
   a.lP = (R*)s.lP;
   a.lQ = (R*)s.lQ;
   a.part = s.part;
@@ -913,6 +981,79 @@ int adjoint_step_impl(lbm_handle* h, const R* fA, const R* gA, const R* JA, int6
   a.walls = p.walls;
   a.u_top = (R)(p.walls ? p.u_wall_top : 0.0);
   a.u_bot = (R)(p.walls ? p.u_wall_bottom : 0.0);
+  return a;
+}
+
+// Whether a sweep of `count` steps takes the chip-resident kernel: the grid
+// fits, and the stream is not being captured (a replay would reuse its tags).
+bool use_sweep(const lbm_handle* h, int32_t count, int64_t stride_bytes) {
+  if (h->adj_res.variant < 0 || count < 2 || stride_bytes % (int64_t)sizeof(float) != 0)
+    return false;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return st == cudaStreamCaptureStatusNone;
+}
+
+// `count` adjoint steps over recorded states, chunks of one launch each.
+int run_sweep(lbm_handle* h, const float* states, int64_t stride, int32_t count, float* adj) {
+  constexpr int32_t kChunk = 4096;
+  AdScratch s = carve(h);
+  const AdArgs<float> a = ad_args<float>(h, s, 0);
+  const lbmk::ResTile* tiles = s.tiles;
+  while (count > 0) {
+    const int32_t cnt = count < kChunk ? count : kChunk;
+    if (h->adj_epoch > UINT32_MAX - 2 * kChunk) {  // tags run out: start over
+      const cudaError_t e =
+          cudaMemsetAsync(s.slots, 0, (size_t)2 * h->adj_res.nslots * sizeof(uint4), h->stream);
+      if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
+      h->adj_epoch = 1;
+    }
+    AdRun r{};
+    r.states = states + (int64_t)(count - cnt) * stride;
+    r.stride = stride;
+    r.count = cnt;
+    r.epoch = h->adj_epoch;
+    r.nslots = h->adj_res.nslots;
+    r.slots = s.slots;
+    r.adj = adj;
+    r.wait_cycles = h->wait_cycles;
+    r.flags = h->flags;
+    h->adj_epoch += (uint32_t)cnt;
+    void* params[] = {(void*)&a, (void*)&tiles, (void*)&r};
+    const cudaError_t e = cudaLaunchCooperativeKernel(
+        (const void*)ad_resident, dim3((unsigned)h->adj_res.tiles.size()), dim3(kAdNT), params,
+        AdShape::SMEM_BYTES, h->stream);
+    if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
+    count -= cnt;
+  }
+  return LBM_OK;
+}
+
+// One adjoint step from the state S_t held in (fA, gA, JA) with plane stride
+// P at step index t (the handle's own buffers, or a snapshot).
+// phase_ready: phi and psi of S_t are already in the scratch planes (the
+// previous step of a sweep formed them); gB/PB: g planes of the state of the
+// next step of a sweep, whose phi and psi the gather launch forms, or null.
+template <typename R>
+int adjoint_step_impl(lbm_handle* h, const R* fA, const R* gA, const R* JA, int64_t P, int64_t t,
+                      const void* d_adj_in, void* d_adj_out, double* h_param_grads,
+                      bool phase_ready = false, const R* gB = nullptr, int64_t PB = 0) {
+  const lbm_params& p = h->params[0];
+  const bool coupled = h->flow == LBM_FLOW_COUPLED;
+  AdScratch s = carve(h);
+  if (!phase_ready)
+    ad_phase<R><<<kAdBlocks, kAdThreads, 0, h->stream>>>(gA, P, p.nx, p.ny, p.walls, (R)p.xi,
+                                                         (R*)s.phi, (R*)s.psi);
+  AdArgs<R> a = ad_args<R>(h, s, t);
+  a.fA = coupled ? fA : nullptr;
+  a.gA = gA;
+  a.JA = JA;
+  a.P = P;
+  a.ain = (const R*)d_adj_in;
+  a.aout = (R*)d_adj_out;
   if (!coupled) {  // the f planes and the tau_f entry stay zero
     cudaError_t e = cudaMemsetAsync(d_adj_out, 0, 9 * sizeof(R) * p.nx * (size_t)p.ny, h->stream);
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
@@ -1009,6 +1150,9 @@ int lbm_adjoint_sweep(lbm_handle* h, const void* d_states, int64_t stride_bytes,
   const size_t es = elem_bytes(h);
   if (count > 1 && stride_bytes < (int64_t)(20 * n * es))
     return fail(LBM_ERR_ARG, "stride_bytes smaller than a state");
+  if (use_sweep(h, count, stride_bytes))
+    return run_sweep(h, (const float*)d_states, stride_bytes / (int64_t)sizeof(float), count,
+                     (float*)d_adj);
   void* cur = d_adj;
   void* nxt = d_spare;
   // each gather launch also forms phi and psi of the state of the next step

@@ -97,4 +97,6 @@ struct lbm_handle {
   // reverse mode (lbm_adjoint_attach): caller-provided FP64 scratch
   char* adj_ws = nullptr;
   size_t adj_ws_bytes = 0;
+  lbmk::ResPlan adj_res;       // tiles of the chip-resident sweep, if the grid fits
+  uint32_t adj_epoch = 1;
 };

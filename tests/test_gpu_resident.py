@@ -119,3 +119,58 @@ def test_recorded_states_are_the_snapshots(L, prec, kind):
         assert float((rec[k] - want).abs().max()) <= tol, k
         b.step(1)
     assert a.status() == L.LBM_OK
+
+
+@pytest.mark.parametrize("walls", [True, False], ids=["walls", "periodic"])
+@pytest.mark.parametrize("nx,ny", [(20, 3), (67, 5), (128, 64), (201, 101), (512, 256)])
+@pytest.mark.parametrize("count", [2, 9])
+def test_reverse_sweep_matches_single_steps(L, nx, ny, walls, count):
+    # one launch over recorded states against lbm_adjoint_step_from step by step.  The arithmetic
+    # is the same up to the contraction of multiply-adds, an ulp (2^-23) of each of the sums that a
+    # step adds up, tens of them: 1e-5 over nine steps.  Parameter sums differ in order as well.
+    import torch
+    from paper_2505_10899_gb300 import adjoint
+    kw = dict(walls=1, u_top=0.02, u_bot=-0.01) if walls else {}
+    case = W.base_case(nx, ny, sigma=5e-3, rho_l=2.0, tau_f_l=0.8, tau_f_g=0.8, **kw)
+    phi0 = 0.5 + 0.3 * np.sin(np.arange(nx) * 2 * np.pi / nx)[None, :] * np.ones((ny, 1))
+    phi0 = phi0 + W.uniform(4, (ny, nx), -0.1, 0.1)
+    a = adjoint.AdjointSim(case, phi0, W.uniform(5, (2, ny, nx), -0.01, 0.01), "f32")
+    a.step(3)
+    rec = torch.empty((count, a.planes) + a.shape, dtype=a.dtype, device="cuda")
+    L.lbm_record_steps(a.h, count, rec.data_ptr(), rec[0].numel() * 4)
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    lam = torch.randn((20, ny, nx), generator=gen, device="cuda")
+    got, spare = lam.clone(), torch.empty_like(lam)
+    L.lbm_adjoint_sweep(a.h, rec.data_ptr(), rec[0].numel() * 4, 3, count, got.data_ptr(),
+                        spare.data_ptr())
+    g1, g2 = np.zeros(6), np.zeros(6)
+    a.take_grads(g1)
+    want = lam
+    for j in range(count - 1, -1, -1):
+        want = a.vjp_step_from(rec[j], 3 + j, want)
+    a.take_grads(g2)
+    assert a.sim.status() == L.LBM_OK
+    assert float((got - want).norm() / want.norm()) <= 1e-5
+    assert float((got - want).abs().max() / want.abs().max()) <= 1e-5
+    assert np.abs(g1 - g2).max() <= 1e-4 * np.abs(g2).max()
+
+
+def test_reverse_sweep_wait_limit(L):
+    # at 0 cycles a CTA whose neighbours' rims have not come at its first poll gives up; the status
+    # is reported once and the sweep runs again from its inputs
+    import torch
+    from paper_2505_10899_gb300 import adjoint
+    case = W.base_case(128, 64)
+    a = adjoint.AdjointSim(case, W.tanh_disc(128, 64, 64.3, 32.2, 16, 4.0, True), None, "f32")
+    rec = torch.empty((8, a.planes) + a.shape, dtype=a.dtype, device="cuda")
+    L.lbm_record_steps(a.h, 8, rec.data_ptr(), rec[0].numel() * 4)
+    lam = torch.ones((20, 64, 128), device="cuda")
+    out = []
+    for limit in (-1, 0, -1):
+        L.lbm_set_wait_limit(a.h, limit)
+        x, spare = lam.clone(), torch.empty_like(lam)
+        L.lbm_adjoint_sweep(a.h, rec.data_ptr(), rec[0].numel() * 4, 0, 8, x.data_ptr(),
+                            spare.data_ptr())
+        assert a.sim.status() == (L.LBM_ERR_TIMEOUT if limit == 0 else L.LBM_OK)
+        out.append(x)
+    assert torch.equal(out[0], out[2])
