@@ -279,7 +279,8 @@ int32_t lbm_num_regions(const lbm_handle* h);
 
 /* Macroscopic fields of case c at the current time, each [ny][nx] FP64:
  * phi (Eq. 35), u (Eq. 28, or the prescribed velocity), p (Eq. 29, 0 in
- * vortex mode).  Any pointer may be NULL.  Synchronises. */
+ * vortex mode).  Any pointer may be NULL, and any may be device memory.
+ * Synchronises. */
 int lbm_fields(lbm_handle* h, int32_t c, double* h_phi, double* h_ux,
                double* h_uy, double* h_p);
 

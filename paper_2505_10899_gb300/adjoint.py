@@ -32,20 +32,30 @@ class AdjointSim:
         self.case = dict(case)
         self.precision = precision
         self.dtype = torch.float64 if precision == "f64" else torch.float32
-        self.sim = lbm.Sim(case, phi0, u0, precision=precision)
-        self.h = self.sim.h
-        self.dev = self.sim.device
         ny, nx = case["ny"], case["nx"]
         self.shape = (ny, nx)
+        # the initial fields (arrays or tensors) as FP64 on the device, once:
+        # lbm_init reads them there, and so does the adjoint of the initial map
+        dev = torch.device("cuda", torch.cuda.current_device())
+
+        def field(a, count):
+            a = a if isinstance(a, torch.Tensor) else torch.from_numpy(
+                np.ascontiguousarray(a, dtype=np.float64))
+            if a.numel() < count:
+                raise ValueError(f"initial field of {a.numel()} values, {count} needed")
+            return a.detach().to(device=dev, dtype=torch.float64, copy=True).contiguous()
+
+        self.phi0 = field(phi0, nx * ny)
+        self.u0 = None if u0 is None else field(u0, 2 * nx * ny)
+        self.sim = lbm.Sim(case, self.phi0.data_ptr(),
+                           None if u0 is None else self.u0.data_ptr(), precision=precision)
+        self.h = self.sim.h
+        self.dev = self.sim.device
         self.planes = lbm.lbm_snapshot_bytes(self.h, 0) // (self.dtype.itemsize * nx * ny)
         nb = lbm.lbm_adjoint_workspace_bytes(self.h)
         self._scratch = torch.empty(nb + 256, dtype=torch.uint8, device=self.dev)
         ptr = (self._scratch.data_ptr() + 255) // 256 * 256
         lbm.lbm_adjoint_attach(self.h, ptr, nb)
-        self.phi0 = torch.as_tensor(np.ascontiguousarray(phi0), dtype=torch.float64,
-                                    device=self.dev)
-        self.u0 = None if u0 is None else torch.as_tensor(np.ascontiguousarray(u0),
-                                                          dtype=torch.float64, device=self.dev)
 
     def new_state(self):
         return torch.zeros((20,) + self.shape, dtype=self.dtype, device=self.dev)
@@ -68,10 +78,12 @@ class AdjointSim:
         return lbm.lbm_time(self.h)
 
     def phi(self):
-        return torch.as_tensor(self.sim.fields(0)[0], device=self.dev)
+        out = torch.empty(self.shape, dtype=torch.float64, device=self.dev)
+        lbm.lbm_field_phi(self.h, 0, out.data_ptr())
+        return out
 
     def seed_phi(self, dphi):
-        adj = self.new_state()
+        adj = torch.empty((20,) + self.shape, dtype=self.dtype, device=self.dev)
         dphi = dphi.to(device=self.dev, dtype=torch.float64).contiguous()
         lbm.lbm_adjoint_seed_phi(self.h, dphi.data_ptr(), adj.data_ptr())
         return adj
@@ -133,7 +145,7 @@ class CoupledRun(torch.autograd.Function):
     @staticmethod
     def forward(ctx, phi0, theta, case, nsteps, ckpt_every, u0, store_bytes, tune, precision):
         th = theta.detach().cpu().numpy().astype(np.float64)
-        asim = AdjointSim(case_with(case, th), phi0.detach().cpu().numpy(), u0, precision)
+        asim = AdjointSim(case_with(case, th), phi0, u0, precision)
         if (nsteps >= 1000) if tune is None else bool(tune):
             asim.sim.autotune(1)  # the forward and the recomputation step with the fastest kernel
         state_bytes = lbm.lbm_snapshot_bytes(asim.h, 0)

@@ -600,6 +600,7 @@ void drop_graph(lbm_handle* h) {
 int capture_steps(lbm_handle* h, int parity, int count, bool flip, bool vol, bool clock,
                   cudaGraphExec_t* out) {
   *out = nullptr;
+  if (!h->cap) LBM_CUDA(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
   LBM_CUDA(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
   int rc = enqueue_steps(h, h->cap, parity, count, flip, vol, clock);
   cudaGraph_t g = nullptr;
@@ -741,7 +742,7 @@ int do_fields(lbm_handle* h, int c, double* phi, double* ux, double* uy, double*
   double* outs[4] = {phi, ux, uy, p};
   for (int q = 0; q < 4; ++q)
     if (outs[q])
-      LBM_CUDA(cudaMemcpyAsync(outs[q], st + q * n, n * sizeof(double), cudaMemcpyDeviceToHost,
+      LBM_CUDA(cudaMemcpyAsync(outs[q], st + q * n, n * sizeof(double), cudaMemcpyDefault,
                                h->stream));
   LBM_CUDA(cudaStreamSynchronize(h->stream));
   return LBM_OK;
@@ -976,8 +977,6 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t 
     lbm_destroy(h);
     return code;
   };
-  if (cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess)
-    return cleanup(fail(LBM_ERR_CUDA, "cannot create capture stream"));
   if (ncases > 1) {  // chains need a stream and an event each (one case: one chain)
     for (int c = 0; c < lbmk::kMaxChains - 1; ++c)
       if (cudaStreamCreateWithFlags(&h->aux[c], cudaStreamNonBlocking) != cudaSuccess ||
@@ -986,7 +985,7 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t 
     if (cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming) != cudaSuccess)
       return cleanup(fail(LBM_ERR_CUDA, "cannot create chain events"));
   }
-  {
+  if (h->tma_ok) {  // handles without the bulk-copy kernel need no attributes of it
     cudaError_t e = h->precision == LBM_F32 ? lbmk::prepare_tma<float>() : lbmk::prepare_tma<double>();
     if (e != cudaSuccess)
       return cleanup(fail(LBM_ERR_CUDA, std::string("kernel attributes: ") + cudaGetErrorString(e)));

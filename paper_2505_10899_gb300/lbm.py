@@ -315,6 +315,12 @@ def lbm_fields(h, c: int, shape):
     return phi, ux, uy, p
 
 
+def lbm_field_phi(h, c: int, out: int):
+    """phi alone (lbm_fields) into [ny][nx] FP64 at address ``out``, host or device memory."""
+    return _check(_lib.lbm_fields(h, int(c), ctypes.cast(ctypes.c_void_p(int(out)), _D), None,
+                                  None, None), "lbm_fields")
+
+
 def lbm_get_state(h, c: int, shape, coupled=True):
     ny, nx = shape
     f = np.zeros((9, ny, nx)) if coupled else None
