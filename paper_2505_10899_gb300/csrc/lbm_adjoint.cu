@@ -1015,6 +1015,7 @@ int run_sweep(lbm_handle* h, const float* states, int64_t stride, int32_t count,
     r.states = states + (int64_t)(count - cnt) * stride;
     r.stride = stride;
     r.count = cnt;
+    r.prefetch = (int64_t)cnt * stride * (int64_t)sizeof(float) > (int64_t)64 << 20;
     r.epoch = h->adj_epoch;
     r.nslots = h->adj_res.nslots;
     r.slots = s.slots;

@@ -174,7 +174,7 @@ __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T
   const T xi = a.ph.xi;
   const bool do_vol = (MODE == kModeStep) && (a.vol_part != nullptr);
   double vacc = 0.0;
-  const CaseK<T> K = case_consts<T, COUPLED>(a, cdp, xc);
+  CaseK<T> K = case_consts<T, COUPLED>(a, cdp, xc);
 
   auto rowoff = [&](int r) -> uint32_t { return (uint32_t)r * (uint32_t)nx; };
   const uint32_t nn = (uint32_t)nx * (uint32_t)ny;  // nodes of the case (checked build)
@@ -289,8 +289,9 @@ __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T
       if (COUPLED && walls && (y == 0 || y == ny - 1))
         wall_momentum(C.F, K.rho_g + S.p * K.drho, y == 0, y == ny - 1, cdp->u_bot,
                       cdp->u_top);
+      if (!COUPLED) vortex_row(K, y);
       const NodeOut<T> o =
-          node_update<T, COUPLED, MODE>(a.ph, K, C.F, C.G, C.lo, C.J[0], C.J[1], S, y);
+          node_update<T, COUPLED, MODE>(a.ph, K, C.F, C.G, C.lo, C.J[0], C.J[1], S);
       const uint32_t node = rowoff(y) + (uint32_t)xc;
       if (MODE == kModeStep) {
         store_node<T, COUPLED>(fd, gd, Jd, lod, P, node, C.F, C.G, C.lo, o, a.flags, nn);

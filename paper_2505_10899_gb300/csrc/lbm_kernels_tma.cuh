@@ -108,7 +108,7 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a) {
   const T xi = a.ph.xi;
   const bool do_vol = (MODE == kModeStep) && (a.vol_part != nullptr);
   double vacc = 0.0;
-  const CaseK<T> K = case_consts<T, COUPLED>(a, cdp, xc);
+  CaseK<T> K = case_consts<T, COUPLED>(a, cdp, xc);
 
   auto wrap = [&](int r) -> int { return r < 0 ? r + ny : (r >= ny ? r - ny : r); };
   auto slot_of = [](int k) -> int { return (k + 1) % S; };
@@ -290,7 +290,8 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a) {
       // fused volume: the plain phi (the low part of g_0, below 2^-24 g_0 per
       // node, is left out here; lbm_volume counts it)
       if (do_vol) vacc += (double)Sn.p;
-      const NodeOut<T> o = node_update<T, COUPLED, MODE>(a.ph, K, F, G, glo, jpx, jpy, Sn, y);
+      if (!COUPLED) vortex_row(K, y);
+      const NodeOut<T> o = node_update<T, COUPLED, MODE>(a.ph, K, F, G, glo, jpx, jpy, Sn);
       if (MODE == kModeStep) {
         store_node<T, COUPLED>(fd, gd, Jd, lod, P, node, F, G, glo, o, a.flags,
                                (uint32_t)nx * (uint32_t)ny);

@@ -200,7 +200,16 @@ struct CaseK {
   int ny;
   T ct;        // vortex: U cos(pi t / T)
   T sx2, s2x;  // vortex: sin^2(pi X), sin(2 pi X) of this thread's column
+  T s2y, sy2;  // vortex: sin(2 pi Y), sin^2(pi Y) of the row (vortex_row)
 };
+
+template <typename T>
+__device__ __forceinline__ void vortex_row(CaseK<T>& K, int y) {
+  T sy, cy;
+  Num<T>::sincospi_((T(y) + T(0.5)) / T(K.ny), &sy, &cy);
+  K.s2y = T(2) * sy * cy;
+  K.sy2 = sy * sy;
+}
 
 template <typename T, bool COUPLED>
 __device__ __forceinline__ CaseK<T> case_consts(const StepArgs<T>& a, const CaseDev<T>* cdp,
@@ -214,9 +223,7 @@ __device__ __forceinline__ CaseK<T> case_consts(const StepArgs<T>& a, const Case
   K.hD7 = cdp->hD7;
   K.var_tau = cdp->var_tau != 0;
   K.ny = cdp->ny;
-  K.ct = T(0);
-  K.sx2 = T(0);
-  K.s2x = T(0);
+  K.ct = K.sx2 = K.s2x = K.s2y = K.sy2 = T(0);
   if (!COUPLED) {
     const double t = (double)(*a.t_base + a.t_off);
     K.ct = (T)(cospi(t / a.ph.vT) * a.ph.vU);
@@ -315,7 +322,7 @@ __device__ __forceinline__ void g_unit(const Phys<double>& ph, double (&G)[9], d
 template <typename T, bool COUPLED, int MODE>
 __device__ __forceinline__ NodeOut<T> node_update(const Phys<T>& ph, const CaseK<T>& K,
                                                   T (&Fc)[9], T (&Gc)[9], T& Glo, T jpx,
-                                                  T jpy, const Stencil<T>& S, int y) {
+                                                  T jpy, const Stencil<T>& S) {
   const T phi = S.p;
   // isotropic stencils (Sec. 3.2): grad = (1/3) axis + (1/12) diagonal
   // differences; lap = (2/3) axis + (1/6) diagonal second differences
@@ -386,10 +393,8 @@ __device__ __forceinline__ NodeOut<T> node_update(const Phys<T>& ph, const CaseK
     }
     }  // !unit
   } else {
-    T sy, cy;
-    Num<T>::sincospi_((T(y) + T(0.5)) / T(K.ny), &sy, &cy);
-    o.ux = -K.ct * K.sx2 * (T(2) * sy * cy);
-    o.uy = K.ct * (sy * sy) * K.s2x;
+    o.ux = -K.ct * K.sx2 * K.s2y;
+    o.uy = K.ct * K.sy2 * K.s2x;
   }
 
   o.Jx = phi * o.ux;

@@ -28,10 +28,13 @@
 // while it is being read.  Tags are unique over the handle's launches.
 //
 // Measured, us per step of a long run, against the kernels replayed from a
-// graph: 128x64 1.65 (was 7.6), 201x101 with walls 2.0 (6.0), 512x256 with
-// walls 3.7 (10.9), vortex 256^2 2.3 (8.9), FP64 128x64 14.7 (38).  What bounds
-// it now: the latency of exchange and collision on small tiles (about 1.6 us),
-// instruction issue on full ones, the FP64 pipe in FP64.
+// graph: 128x64 1.58 (was 7.6), 201x101 with walls 1.87 (6.0), 512x256 with
+// walls 3.65 (10.9), vortex 256^2 2.10 (8.9), FP64 128x64 9.6 (38).  What
+// bounds it now: the latency of exchange and collision on small tiles (about
+// 1.6 us; 13% of issue slots), on full ones 540 instructions per node at 45%
+// issue with 16 warps and three barriers per step, the FP64 pipe in FP64.  Two
+// polling loads in flight instead of one changed nothing: most words have
+// come by the first poll.
 //
 // Per step: collide (shared -> shared), barrier, send the rim, form phi and
 // psi of the nodes whose pull needs no rim, receive the rim, barrier, phi and
@@ -282,10 +285,13 @@ __global__ void __launch_bounds__(NT, MINB)
   K.hD7 = cdp->hD7;
   K.var_tau = cdp->var_tau != 0;
   K.ny = ny;
-  K.ct = K.sx2 = K.s2x = T(0);
+  K.ct = K.sx2 = K.s2x = K.s2y = K.sy2 = T(0);
   constexpr bool LO = sizeof(T) == 4;
-  T jx[R], jy[R], lo[R], sx2[R], s2x[R];
+  T jx[R], jy[R], lo[R], sx2[R], s2x[R], s2y[R], sy2[R];
   int cel[R];  // cell of node r, or -1
+  // what the step needs to know of node r, found once: bit 0 no rim needed for
+  // its phi, bits 1, 2 wall row below, above
+  uint32_t kind[R];
   uint32_t gnode[R];
 #pragma unroll
   for (int r = 0; r < R; ++r) {
@@ -293,14 +299,19 @@ __global__ void __launch_bounds__(NT, MINB)
     const bool act = k < w * h;
     const int ly = act ? k / w : 0, lx = act ? k - ly * w : 0;
     cel[r] = act ? cell_of(lx, ly) : -1;
+    kind[r] = ((lx >= 1 && lx <= w - 2 && ly >= 1 && ly <= h - 2) ? 1u : 0u) |
+              ((wbot && ly == 0) ? 2u : 0u) | ((wtop && ly == h - 1) ? 4u : 0u);
     const uint32_t node = (uint32_t)(tl.y0 + ly) * (uint32_t)nx + (uint32_t)(tl.x0 + lx);
     gnode[r] = node;
     const bool ok = act && LBM_BOUND(a.flags, node, nn);
     jx[r] = ok ? cdp->J[a.parity][node] : T(0);
     jy[r] = ok ? cdp->J[a.parity][P + node] : T(0);
     lo[r] = (LO && ok) ? cdp->g0lo[a.parity][node] : T(0);
-    sx2[r] = s2x[r] = T(0);
+    sx2[r] = s2x[r] = s2y[r] = sy2[r] = T(0);
     if (!COUPLED) {
+      vortex_row(K, tl.y0 + ly);
+      s2y[r] = K.s2y;
+      sy2[r] = K.sy2;
       T s, c;
       Num<T>::sincospi_((T(tl.x0 + lx) + T(0.5)) / T(nx), &s, &c);
       sx2[r] = s * s;
@@ -319,12 +330,16 @@ __global__ void __launch_bounds__(NT, MINB)
     v[0] = o[0];
     v[1] = o[1 * PC - 1];
     v[3] = o[3 * PC + 1];
-    v[2] = bt ? o[4 * PC] : m[2 * PC];
-    v[5] = bt ? o[7 * PC] : m[5 * PC - 1];
-    v[6] = bt ? o[8 * PC] : m[6 * PC + 1];
-    v[4] = tp ? o[2 * PC] : p[4 * PC];
-    v[7] = tp ? o[5 * PC] : p[7 * PC + 1];
-    v[8] = tp ? o[6 * PC] : p[8 * PC - 1];
+    v[2] = m[2 * PC];
+    v[5] = m[5 * PC - 1];
+    v[6] = m[6 * PC + 1];
+    v[4] = p[4 * PC];
+    v[7] = p[7 * PC + 1];
+    v[8] = p[8 * PC - 1];
+    if (COUPLED && (bt || tp)) {
+      if (bt) v[2] = o[4 * PC], v[5] = o[7 * PC], v[6] = o[8 * PC];
+      if (tp) v[4] = o[2 * PC], v[7] = o[5 * PC], v[8] = o[6 * PC];
+    }
   };
   auto phase_a = [&](const T* b, int src, int dst, bool bt, bool tp) {
     T G[9];
@@ -339,9 +354,7 @@ __global__ void __launch_bounds__(NT, MINB)
   auto phase_inner = [&](const T* b) {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      if (cel[r] < 0) continue;
-      const int ly = cel[r] / pw - 2, lx = cel[r] - (ly + 2) * pw - 2;
-      if (lx >= 1 && lx <= w - 2 && ly >= 1 && ly <= h - 2) phase_a(b, cel[r], cel[r], false, false);
+      if (cel[r] >= 0 && (kind[r] & 1u)) phase_a(b, cel[r], cel[r], false, false);
     }
   };
   auto phase_edge = [&](const T* b) {
@@ -385,8 +398,8 @@ __global__ void __launch_bounds__(NT, MINB)
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if (cel[r] < 0) continue;
-      const int c = cel[r], y = tl.y0 + c / pw - 2;
-      const bool bt = walls && y == 0, tp = walls && y == ny - 1;
+      const int c = cel[r];
+      const bool bt = kind[r] & 2u, tp = kind[r] & 4u;
       T F[9], G[9];
       pull(cur, c, bt, tp, G);
       if (COUPLED) pull(cur + (size_t)9 * PC, c, bt, tp, F);
@@ -407,9 +420,11 @@ __global__ void __launch_bounds__(NT, MINB)
         K.ct = ctab[s];
         K.sx2 = sx2[r];
         K.s2x = s2x[r];
+        K.s2y = s2y[r];
+        K.sy2 = sy2[r];
       }
       const NodeOut<T> o =
-          node_update<T, COUPLED, kModeStep>(a.ph, K, F, G, lo[r], jx[r], jy[r], S, y);
+          node_update<T, COUPLED, kModeStep>(a.ph, K, F, G, lo[r], jx[r], jy[r], S);
       jx[r] = o.Jx;
       jy[r] = o.Jy;
 #pragma unroll
