@@ -96,7 +96,7 @@ static cudaError_t launch_strip(const Args3<T, S>& a, cudaStream_t st) {
   }
   if (a.nx % BX != 0) return cudaErrorInvalidValue;
   const dim3 grid(a.nx / BX, (a.ny + BY - 1) / BY, (a.nz + a.zc - 1) / a.zc);
-  step3_strip_kernel<T, S, BX, BY, NST, MINB><<<grid, BX * BY, bytes, st>>>(a, a.wait);
+  step3_strip_kernel<T, S, BX, BY, NST, MINB><<<grid, BX * BY / 2, bytes, st>>>(a, a.wait);
   return cudaGetLastError();
 }
 

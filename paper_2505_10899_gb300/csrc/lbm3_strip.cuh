@@ -36,6 +36,7 @@
 
 #include "lbm3_bulk.cuh"
 #include "lbm3_kernels.cuh"
+#include "lbm3_pair.cuh"
 #include "lbm_tma.cuh"
 
 namespace lbmk3 {
@@ -64,7 +65,6 @@ struct StripShape {
   static constexpr uint32_t TX_BYTES =
       (uint32_t)(((19 * BX + 10 * ES) * BY + (6 * BX + 10 * ES) * NR) * sizeof(S) +
                  (3 * BX * BY + 2 * (BX + 2 * ET) * NR) * sizeof(T));
-  static constexpr int NH = 2 * RW + 2 * BY;  // halo ring of the tile
   static_assert(BX % ES == 0 && BX % ET == 0, "strip width must be whole 16-byte chunks");
   static_assert(ES >= 2 && ET >= 2, "a chunk must cover the pull shift and the halo column");
   static_assert(STAGE_BYTES % 16 == 0 && GM_OFF % 16 == 0 && J_OFF % 16 == 0 &&
@@ -78,7 +78,7 @@ constexpr size_t strip_smem_bytes() {
 }
 
 template <typename T, typename S, int BX, int BY, int NST, int MINB>
-__global__ void __launch_bounds__(BX* BY, MINB)
+__global__ void __launch_bounds__(BX* BY / 2, MINB)
     step3_strip_kernel(const Args3<T, S> a, long long wait_cycles) {
   using SH = StripShape<T, S, BX, BY, NST>;
   using Pair = typename N3<T>::pair;
@@ -88,7 +88,9 @@ __global__ void __launch_bounds__(BX* BY, MINB)
   Pair(*const ring)[NR][RW] = reinterpret_cast<Pair(*)[NR][RW]>(smem + SH::RING_OFF);
 
   const int tid = threadIdx.x;
-  const int tx = tid % BX, ty = tid / BX, warp = tid >> 5, lane = tid & 31;
+  constexpr int NT = BX * BY / 2;
+  // the thread's nodes: columns tx and tx + 1 (tx even) of row ty
+  const int tx = 2 * (tid % (BX / 2)), ty = tid / (BX / 2), warp = tid >> 5, lane = tid & 31;
   const int nx = a.nx, ny = a.ny, nz = a.nz;
   const int64_t P = a.plane;
   const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
@@ -133,17 +135,14 @@ __global__ void __launch_bounds__(BX* BY, MINB)
 
   // Row segments of a stage (local plane k, plane z = zb + k): f and phi*u of
   // the BY rows of plane z, the g of the NR phase-A rows of plane z + 1.
-  // Thread q < NQ copies segment q of every stage.  Its segment is described
+  // Thread q % NT copies segment q of every stage.  A segment is described
   // once per CTA (only the plane changes from stage to stage): piece A's
   // global address without the plane offset, its byte offset inside a stage,
   // its size, the plane it reads (0..3: z-1 .. z+2) and the element size;
   // and, where the segment crosses x = 0 or x = nx (nx >= 2 BX: at most one
   // of the two), piece B's address relative to A, stage offset and size.
-  constexpr int NT = BX * BY;
-  static_assert(SH::NQ <= NT, "one row segment per thread at most");
-  __shared__ uint4 qdesc[2][NT];
-  if (tid < SH::NQ) {
-    const int q = tid;
+  __shared__ uint4 qdesc[2][SH::NQ];
+  for (int q = tid; q < SH::NQ; q += NT) {
     const unsigned char* base;
     int rsel, dz, xa, len, esz;
     size_t dst;
@@ -203,15 +202,16 @@ __global__ void __launch_bounds__(BX* BY, MINB)
     const int z2 = z1 + 1 == nz ? 0 : z1 + 1;
     const int z3 = z2 + 1 == nz ? 0 : z2 + 1;
     if (tid == 0) lbmk::mbar_arrive_expect_tx(bar, SH::TX_BYTES);
-    if (tid < SH::NQ) {
-      const uint4 d0 = qdesc[0][tid];
+#pragma unroll
+    for (int q = tid; q < SH::NQ; q += NT) {
+      const uint4 d0 = qdesc[0][q];
       const uint32_t dz = (d0.w >> 24) & 3u;
       const int zp = dz == 0 ? zq : (dz == 1 ? z1 : (dz == 2 ? z2 : z3));
       const unsigned char* src =
           reinterpret_cast<const unsigned char*>(((uint64_t)d0.y << 32) | d0.x) +
           ((size_t)((uint32_t)zp * nxy) << (d0.w >> 28));
       lbmk::bulk_g2s(st + d0.z, src, d0.w & 0xFFFFFFu, bar);
-      const uint4 d1 = qdesc[1][tid];
+      const uint4 d1 = qdesc[1][q];
       if (d1.z) lbmk::bulk_g2s(st + d1.y, src + (int32_t)d1.x, d1.z, bar);
     }
     zq = z1;
@@ -232,19 +232,33 @@ __global__ void __launch_bounds__(BX* BY, MINB)
     ring[slot][r][xl + 1] = v;
   };
 
-  // Halo position h of the tile (tile coordinates -1..BX, -1..BY): the rows
-  // above and below, then the columns left and right.  Thread tid takes
-  // positions tid, tid + NT, ... (one at most where NH <= NT).
-  auto halo_xy = [&](int h, int& hx, int& hy) {
-    if (h < RW) {
-      hx = h - 1, hy = -1;
-    } else if (h < 2 * RW) {
-      hx = h - RW - 1, hy = BY;
-    } else if (h < 2 * RW + BY) {
-      hx = -1, hy = h - 2 * RW;
-    } else {
-      hx = BX, hy = h - 2 * RW - BY;
-    }
+  // the same at columns xl and xl + 1 (xl even: what is not shifted is one
+  // aligned load)
+  auto staged_g2 = [&](unsigned char* st, int r, int xl, float2 (&G)[7], float2& glo) {
+    G[0] = ld2<0>(sG0(st, 0, r) + xl + ET);
+    glo = ld2<0>(sG0(st, 1, r) + xl + ET);
+    G[1] = ld2<1>(sGM(st, 1, r) + xl + ES);
+    G[2] = ld2<-1>(sGM(st, 2, r) + xl + ES);
+#pragma unroll
+    for (int m = 3; m < 7; ++m) G[m] = ld2<0>(sGM(st, m, r) + xl + ES);
+  };
+  auto put2 = [&](int slot, int r, int xl, const float2 (&G)[7], float2 glo) {
+    const float2 phi = add2(
+        add2(add2(add2(G[0], add2(G[1], G[2])), add2(G[3], G[4])), add2(G[5], G[6])), glo);
+    ring[slot][r][xl + 1] = make_float2(phi.x, psi3(phi.x, a.xi));
+    ring[slot][r][xl + 2] = make_float2(phi.y, psi3(phi.y, a.xi));
+  };
+
+  // The tile's halo ring, tile coordinates -1 .. BX and -1 .. BY: items h < BX
+  // are node pairs of the rows below and above, the others single nodes of
+  // the columns left and right (corners included).
+  constexpr int NHI = BX + 2 * NR;
+  auto halo_pair = [&](int h, int& hx, int& hy) {
+    hx = 2 * (h % (BX / 2)), hy = h < BX / 2 ? -1 : BY;
+  };
+  auto halo_node = [&](int h, int& hx, int& hy) {
+    const int u = h - BX;
+    hx = u < NR ? -1 : BX, hy = (u < NR ? u : u - NR) - 1;
   };
 
   for (int k = 0; k < NST - 1 && k < nplanes; ++k) issue(k);
@@ -252,28 +266,35 @@ __global__ void __launch_bounds__(BX* BY, MINB)
   int landed = -1;
 
   // ---- prologue: phase A of planes zb-1 and zb from global memory ----------
-  T Gc[7], Gn[7], Gcl = T(0), Gnl = T(0);
+  float2 Gc[7], Gn[7], Gcl, Gnl;
   {
-    const uint32_t nxy = (uint32_t)nx * (uint32_t)ny;
-    Offs own;
-    set_xy(own, x0 + tx, wrapy(y0 + ty), nx, ny);
+    auto pull = [&](int x, int y, int zl, T (&G)[7], T& gl) {  // tile coordinates
+      Offs o;
+      set_xy(o, (x0 + x + nx) % nx, wrapy(y0 + y), nx, ny);
+      set_z(o, zl, nz, nxy);
+      pull_g(g0s, g0ls, gms, P, o, G, gl);
+    };
     for (int q = 0; q < 2; ++q) {
-      const int zl = wrapz(zb - 1 + q);
-      set_z(own, zl, nz, nxy);
-      T G[7], gl;
-      pull_g(g0s, g0ls, gms, P, own, G, gl);
-      put((zb - 1 + q) & 3, ty + 1, tx, G, gl);
+      const int zl = wrapz(zb - 1 + q), slot = (zb - 1 + q) & 3;
+      T A[7], B[7], al, bl;
+      pull(tx, ty, zl, A, al);
+      pull(tx + 1, ty, zl, B, bl);
+      put(slot, ty + 1, tx, A, al);
+      put(slot, ty + 1, tx + 1, B, bl);
 #pragma unroll
-      for (int i = 0; i < 7; ++i) (q == 0 ? Gn : Gc)[i] = G[i];
-      (q == 0 ? Gnl : Gcl) = gl;
-      for (int h = tid; h < SH::NH; h += NT) {
+      for (int i = 0; i < 7; ++i) Gc[i] = make_float2(A[i], B[i]);  // of plane zb in the end
+      Gcl = make_float2(al, bl);
+      for (int h = tid; h < NHI; h += NT) {
         int hx, hy;
-        halo_xy(h, hx, hy);
-        Offs hal;
-        set_xy(hal, (x0 + hx + nx) % nx, wrapy(y0 + hy), nx, ny);
-        set_z(hal, zl, nz, nxy);
-        pull_g(g0s, g0ls, gms, P, hal, G, gl);
-        put((zb - 1 + q) & 3, hy + 1, hx, G, gl);
+        if (h < BX) {
+          halo_pair(h, hx, hy);
+          pull(hx + 1, hy, zl, A, al);
+          put(slot, hy + 1, hx + 1, A, al);
+        } else {
+          halo_node(h, hx, hy);
+        }
+        pull(hx, hy, zl, A, al);
+        put(slot, hy + 1, hx, A, al);
       }
     }
   }
@@ -287,14 +308,22 @@ __global__ void __launch_bounds__(BX* BY, MINB)
     if (!bad) {
       landed = k;
       // phase A of plane z + 1 from the staged g rows
-      staged_g(st, ty + 1, tx, Gn, Gnl);
-      put((z + 1) & 3, ty + 1, tx, Gn, Gnl);
-      for (int h = tid; h < SH::NH; h += NT) {
+      staged_g2(st, ty + 1, tx, Gn, Gnl);
+      put2((z + 1) & 3, ty + 1, tx, Gn, Gnl);
+#pragma unroll
+      for (int h = tid; h < NHI; h += NT) {
         int hx, hy;
-        halo_xy(h, hx, hy);
-        T H[7], hl;
-        staged_g(st, hy + 1, hx, H, hl);
-        put((z + 1) & 3, hy + 1, hx, H, hl);
+        if (h < BX) {
+          halo_pair(h, hx, hy);
+          float2 H[7], hl;
+          staged_g2(st, hy + 1, hx, H, hl);
+          put2((z + 1) & 3, hy + 1, hx, H, hl);
+        } else {
+          halo_node(h, hx, hy);
+          T H[7], hl;
+          staged_g(st, hy + 1, hx, H, hl);
+          put((z + 1) & 3, hy + 1, hx, H, hl);
+        }
       }
     }
     if (__syncthreads_or(bad)) {
@@ -313,40 +342,47 @@ __global__ void __launch_bounds__(BX* BY, MINB)
       issued_last = nxt;
     }
     if (act) {
-      T F[19], jp[3];
+      float2 F[19], jp[3];
 #pragma unroll
-      for (int i = 0; i < 19; ++i) F[i] = Conv<T, S>::ld(sF(st, i, ty) + (tx - bcx(i) + ES));
+      for (int i = 0; i < 19; ++i) {
+        const S* const q = sF(st, i, ty) + tx + ES;
+        F[i] = bcx(i) == 0 ? ld2<0>(q) : (bcx(i) == 1 ? ld2<1>(q) : ld2<-1>(q));
+      }
 #pragma unroll
-      for (int c = 0; c < 3; ++c) jp[c] = sJ(st, c, ty)[tx];
-      // stencils of plane z from the ring: planes z-1, z, z+1, rows ty..ty+2
-      const int sm = (z + 3) & 3, s0 = z & 3, sp = (z + 1) & 3, j = ty + 1, i = tx + 1;
-      const Pair c = ring[s0][j][i], e = ring[s0][j][i + 1], w = ring[s0][j][i - 1];
-      const Pair n = ring[s0][j + 1][i], s = ring[s0][j - 1][i];
-      const Pair ne = ring[s0][j + 1][i + 1], nw = ring[s0][j + 1][i - 1];
-      const Pair se = ring[s0][j - 1][i + 1], sw = ring[s0][j - 1][i - 1];
-      const Pair u = ring[sp][j][i], ue = ring[sp][j][i + 1], uw = ring[sp][j][i - 1];
-      const Pair un = ring[sp][j + 1][i], us = ring[sp][j - 1][i];
-      const Pair d = ring[sm][j][i], de = ring[sm][j][i + 1], dw = ring[sm][j][i - 1];
-      const Pair dn = ring[sm][j + 1][i], ds = ring[sm][j - 1][i];
-      const St3<T> SP{c.x, e.x, w.x, n.x, s.x, ne.x, nw.x, se.x, sw.x, u.x, ue.x, uw.x,
-                      un.x, us.x, d.x, de.x, dw.x, dn.x, ds.x};
-      const St3<T> SQ{c.y, e.y, w.y, n.y, s.y, ne.y, nw.y, se.y, sw.y, u.y, ue.y, uw.y,
-                      un.y, us.y, d.y, de.y, dw.y, dn.y, ds.y};
-      const Out3<T> o = node3<T, S, kModeStep>(a, F, Gc, Gcl, jp, SP, SQ);
-      const T phi = SP.C;
-      if (!(isfinite(phi) && isfinite(o.ux + o.uy + o.uz))) atomicOr(a.flags, kFlagNonFinite);
-      if (a.vol_part) vsum += (double)phi;
+      for (int c = 0; c < 3; ++c) jp[c] = ld2<0>(sJ(st, c, ty) + tx);
+      Pair2 N;
+      {
+        // (phi, psi) of columns tx-1 .. tx+2, rows ty-1 .. ty+1, planes z-1 .. z+1
+        const int sm = (z + 3) & 3, s0 = z & 3, sp = (z + 1) & 3, j = ty + 1;
+        float2 C[4], Nr[4], Sr[4], U[4], D[4], un[2], us[2], dn[2], ds[2];
+        row4(&ring[s0][j][tx], C);
+        row4(&ring[s0][j + 1][tx], Nr);
+        row4(&ring[s0][j - 1][tx], Sr);
+        row4(&ring[sp][j][tx], U);
+        row4(&ring[sm][j][tx], D);
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+          un[n] = ring[sp][j + 1][tx + 1 + n];
+          us[n] = ring[sp][j - 1][tx + 1 + n];
+          dn[n] = ring[sm][j + 1][tx + 1 + n];
+          ds[n] = ring[sm][j - 1][tx + 1 + n];
+        }
+        stencils2(C, Nr, Sr, U, D, un, us, dn, ds, N);
+      }
+      float2 J[3];
+      const float2 fin = node3_pair<S>(a, F, Gc, Gcl, jp, N, J);
+      if (!(isfinite(fin.x) && isfinite(fin.y))) atomicOr(a.flags, kFlagNonFinite);
+      if (a.vol_part) vsum += (double)N.phi.x + (double)N.phi.y;
       const uint32_t node = ((uint32_t)z * (uint32_t)ny + (uint32_t)(y0 + ty)) * (uint32_t)nx +
                             (uint32_t)(x0 + tx);
-      jd[node] = phi * o.ux;
-      jd[P + node] = phi * o.uy;
-      jd[2 * P + node] = phi * o.uz;
-      g0d[node] = Gc[0];
-      g0ld[node] = Gcl;
 #pragma unroll
-      for (int m = 1; m < 7; ++m) gmd[(m - 1) * P + node] = Conv<T, S>::st(Gc[m]);
+      for (int c = 0; c < 3; ++c) *reinterpret_cast<float2*>(jd + c * P + node) = J[c];
+      *reinterpret_cast<float2*>(g0d + node) = Gc[0];
+      *reinterpret_cast<float2*>(g0ld + node) = Gcl;
 #pragma unroll
-      for (int q = 0; q < 19; ++q) fd[q * P + node] = Conv<T, S>::st(F[q]);
+      for (int m = 1; m < 7; ++m) st2(gmd + (m - 1) * P + node, Gc[m]);
+#pragma unroll
+      for (int q = 0; q < 19; ++q) st2(fd + q * P + node, F[q]);
     }
 #pragma unroll
     for (int m = 0; m < 7; ++m) Gc[m] = Gn[m];
@@ -356,12 +392,12 @@ __global__ void __launch_bounds__(BX* BY, MINB)
     // fixed-order block reduction of the phi this CTA collided
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) vsum += __shfl_down_sync(0xffffffffu, vsum, off);
-    __shared__ double wsum[BX * BY / 32];
+    __shared__ double wsum[NT / 32];
     if (lane == 0) wsum[warp] = vsum;
     __syncthreads();
     if (tid == 0) {
       double t = 0.0;
-      for (int w = 0; w < BX * BY / 32; ++w) t += wsum[w];
+      for (int w = 0; w < NT / 32; ++w) t += wsum[w];
       a.vol_part[((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = t;
     }
   }
