@@ -129,7 +129,8 @@ int lbm3_set_tiling(lbm3_handle* h, int32_t bx, int32_t by, int32_t zc);
 int lbm3_get_tiling(const lbm3_handle* h, int32_t* bx, int32_t* by, int32_t* zc,
                     int32_t* n_ctas);
 
-/* Step-kernel variant.  All variants run the same per-node arithmetic.
+/* Step-kernel variant.  All variants solve the same equations (variants 5 and
+ * 6 in a shorter form: equal up to rounding).
  *   0: automatic -- the register kernel until lbm3_autotune picks the
  *      fastest (on a tile the register kernel does not run, with the
  *      default tile (32, 8));
@@ -142,9 +143,9 @@ int lbm3_get_tiling(const lbm3_handle* h, int32_t* bx, int32_t* by, int32_t* zc,
  *      stored values and of nx FP32 values a multiple of 16 bytes; tiles
  *      (128, 4) for nx <= 128, (256, 2); selecting it on another tile takes
  *      its own tile);
- *   5: bulk copies of padded row segments of a bx-column strip (one 16-byte
- *      chunk each side for the pull's shift and the halo column; split where
- *      they cross the periodic edge), two (FP32) or three (FP16) stages
+ *   5: asynchronous 16-byte copies of the padded rows of a bx-column strip
+ *      (one chunk each side for the pull's shift and the halo column), two
+ *      nodes per thread in packed arithmetic, two (FP32) or three (FP16) stages
  *      deep, two CTAs per SM (LBM3_F32 and LBM3_F16; nx a multiple of bx and
  *      nx >= 2 bx; tiles (32, 8), (64, 4); selecting it on another tile takes
  *      (64, 4) where nx allows, else (32, 8));

@@ -112,7 +112,7 @@ static cudaError_t step_async(const Args3<T, S>& a, int variant, int bx, int by,
       return cudaErrorInvalidValue;
     }
     if (variant == kVarStrip) {
-      // about 90 KB per CTA of 256 threads: two CTAs per SM, with three FP16
+      // about 90 KB per CTA of 128 threads: two CTAs per SM, with three FP16
       // stages or two FP32 ones per CTA
       constexpr int NST = sizeof(S) == 2 ? 3 : 2;
       if (bx == 32 && by == 8) return launch_strip<T, S, 32, 8, NST, 2>(a, st);
@@ -120,7 +120,7 @@ static cudaError_t step_async(const Args3<T, S>& a, int variant, int bx, int by,
       return cudaErrorInvalidValue;
     }
     if (variant == kVarStripOcc) {
-      // two stages per CTA and at most 80 (64 x 4) or 96 (64 x 2) registers:
+      // two stages per CTA and at most 168 (64 x 4) or 204 (64 x 2) registers:
       // three or five CTAs per SM where shared memory allows (FP16 storage)
       if (bx == 64 && by == 4) return launch_strip<T, S, 64, 4, 2, 3>(a, st);
       if (bx == 64 && by == 2) return launch_strip<T, S, 64, 2, 2, 5>(a, st);

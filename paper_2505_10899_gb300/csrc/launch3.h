@@ -33,7 +33,7 @@ inline bool tile_regs_ok(int bx, int by) {
 }
 // Tiles of the bulk-copy kernel: whole x-rows, 128 x 4 or 256 x 2.
 inline bool tile_bulk_ok(int bx, int by) { return (bx == 128 && by == 4) || (bx == 256 && by == 2); }
-// Tiles of the strip bulk-copy kernel (nx a multiple of bx, nx >= 2 bx).
+// Tiles of the strip kernel (nx a multiple of bx, nx >= 2 bx).
 inline bool tile_strip_ok(int bx, int by) { return (bx == 32 && by == 8) || (bx == 64 && by == 4); }
 // Tiles of the strip kernel's occupancy form (two stages, more CTAs per SM).
 inline bool tile_strip_occ_ok(int bx, int by) { return bx == 64 && (by == 4 || by == 2); }
@@ -50,10 +50,10 @@ inline int64_t n_ctas(int nx, int ny, int nz, int bx, int by, int zc) {
 // asynchronous copies through shared memory with 2 or 3 stages (FP32 only);
 // bulk copies of whole rows into shared memory (FP32 arithmetic, FP32 or
 // FP16 storage; rows of nx <= bx values, nx values a multiple of 16 bytes);
-// bulk copies of padded strip-row segments (FP32 arithmetic, FP32 or FP16
-// storage; nx a multiple of bx and at least two strips), with two or three
-// stages and two CTAs per SM (5), or two stages and three (64 x 4) or five
-// (64 x 2) CTAs per SM at fewer registers (6).
+// 16-byte copies of padded strip rows, two nodes per thread (FP32 arithmetic,
+// FP32 or FP16 storage; nx a multiple of bx and at least two strips), with two
+// or three stages and two CTAs per SM (5), or two stages and three (64 x 4) or
+// five (64 x 2) CTAs per SM at fewer registers (6).
 enum { kVarRegs = 1, kVarAsync2 = 2, kVarAsync3 = 3, kVarBulk = 4, kVarStrip = 5,
        kVarStripOcc = 6 };
 

@@ -28,7 +28,7 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {  // one rounding, as a - b
-  return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a);
+  return __fadd2_rn(a, make_float2(-b.x, -b.y));
 }
 
 // Values at p - CX and p + 1 - CX (p even: without a shift one aligned load).

@@ -1,14 +1,13 @@
-// Strip-tiled bulk-copy variant of the three-dimensional step kernel (FP32
+// Strip-tiled staged variant of the three-dimensional step kernel (FP32
 // arithmetic, FP32 or FP16 population storage) for boxes whose nx is a
-// multiple of the strip width BX and at least 2 BX.  Same per-node
-// arithmetic as step3_kernel (node3, the same stencils and phase-A sums); the
-// difference is how the pulled values reach the threads.
+// multiple of the strip width BX and at least 2 BX.  The equations of
+// step3_kernel; the difference is how the pulled values reach the threads, and
+// that a thread updates two nodes adjacent in x at a time (lbm3_pair.cuh).
 //
 // A CTA owns a BX x BY column tile (x0 .. x0+BX-1, y0 .. y0+BY-1) and marches
 // along z over `zc` planes, like step3_kernel, so several CTAs share an SM.
-// Every value it reads for plane z arrives in shared memory by 1-D bulk
-// copies (cp.async.bulk) of row segments, one segment per thread of the CTA,
-// NST-1 planes ahead, completed on one mbarrier per stage:
+// Every value it reads for plane z arrives in shared memory by asynchronous
+// 16-byte copies, NST-1 planes ahead, counted on one mbarrier per stage:
 //   - f_i: row (y - c_iy, z - c_iz) of plane i for each of the BY rows, over
 //     columns x0 .. x0+BX-1 shifted by -c_ix;
 //   - phi*u: rows (y, z), columns x0 .. x0+BX-1;
@@ -18,13 +17,25 @@
 //     from which the D3Q19 stencils of Sec. 3.2 are read.
 // A staged row starts one 16-byte chunk (ES stored values, or ET values of
 // the arithmetic type for the g_0 rows) left of x0 and ends one chunk right
-// of x0+BX-1, so that the pull's one-column shift and the halo
-// columns are index offsets inside it; a segment copies only the chunks its
-// population reads (no left chunk for c_x = -1 rows of f, and so on).  Where a
-// segment crosses the periodic edge x = 0 or x = nx it is split there (nx is
-// a multiple of the chunk, so every piece stays 16-byte aligned).  The pulled
-// g of a thread's own node stay in registers from phase A (plane z+1) to the
+// of x0+BX-1, so that the pull's one-column shift and the halo columns are
+// index offsets inside it; of the two outer chunks only those its population
+// reads are copied, from the other end of the row at x = 0 and x = nx (nx is
+// a multiple of the chunk, so every copy stays 16-byte aligned).  The pulled g
+// of a thread's own nodes stay in registers from phase A (plane z+1) to the
 // update of plane z+1.
+//
+// Why threads copy and not the bulk engine: a row is 128 to 288 bytes, and a
+// plane's 136 to 198 row segments were as many bulk-copy instructions, which
+// take their operands from uniform registers, so a warp issues them lane after
+// lane (the profiler counted 198 of them and 23.7 active threads per
+// instruction).  A thread's 11 (FP16) or 18 (FP32) chunk copies are 128-thread
+// wide.  Per node 703 -> 557 instructions in FP16 storage, 642 -> 532 in FP32.
+// Measured, 256 x 256 x 512, MLUPS, bulk copies -> chunk copies: FP16 64 x 4 x
+// 32 with three CTAs per SM 31,300 -> 38,470 (0.73 of measured HBM), 64 x 2 x
+// 64 25,270 -> 34,450, with three stages and two CTAs 24,930 -> 34,530; FP32
+// 64 x 4 x 64 22,060 -> 24,290 (0.83).  One node per thread, not packed, with
+// bulk copies: FP16 28,300, FP32 22,200.  What bounds it now: HBM in FP32; in
+// FP16 issue (51%) and the latency of shared loads at 12 warps per SM.
 //
 // Every wait is bounded (wait_cycles); on expiry the CTA raises
 // kFlagTimeout3, waits (bounded by lbmk::kWaitCycles) for its own copies in
@@ -58,13 +69,9 @@ struct StripShape {
   static constexpr size_t RING_OFF = (BAR_OFF + NST * 8 + 127) / 128 * 128;
   static constexpr size_t RING_BYTES = (size_t)4 * NR * RW * sizeof(typename N3<T>::pair);
   static constexpr size_t SMEM_BYTES = RING_OFF + RING_BYTES;
-  static constexpr int NQ = 22 * BY + 8 * NR;  // row segments per stage
-  // bytes one stage receives: five f rows per tile row carry a left chunk and
-  // five a right chunk; of the six g movers one has no left chunk and one no
-  // right chunk; g_0 and its low part carry both
-  static constexpr uint32_t TX_BYTES =
-      (uint32_t)(((19 * BX + 10 * ES) * BY + (6 * BX + 10 * ES) * NR) * sizeof(S) +
-                 (3 * BX * BY + 2 * (BX + 2 * ET) * NR) * sizeof(T));
+  static constexpr int NROW_S = 19 * BY + 6 * NR;          // rows of stored values per stage
+  static constexpr int NROW = NROW_S + 3 * BY + 2 * NR;    // and of the arithmetic type
+  static constexpr int NPAD = 10 * BY + 10 * NR + 4 * NR;  // chunks left and right of them
   static_assert(BX % ES == 0 && BX % ET == 0, "strip width must be whole 16-byte chunks");
   static_assert(ES >= 2 && ET >= 2, "a chunk must cover the pull shift and the halo column");
   static_assert(STAGE_BYTES % 16 == 0 && GM_OFF % 16 == 0 && J_OFF % 16 == 0 &&
@@ -129,91 +136,101 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
     return reinterpret_cast<T*>(st + SH::G0_OFF) + ((size_t)h * NR + r) * WT;
   };
   if (tid == 0) {
-    for (int s = 0; s < NST; ++s) lbmk::mbar_init(&bars[s], 1);
+    for (int s = 0; s < NST; ++s) lbmk::mbar_init(&bars[s], NT);
     lbmk::fence_mbar_init();
   }
 
-  // Row segments of a stage (local plane k, plane z = zb + k): f and phi*u of
-  // the BY rows of plane z, the g of the NR phase-A rows of plane z + 1.
-  // Thread q % NT copies segment q of every stage.  A segment is described
-  // once per CTA (only the plane changes from stage to stage): piece A's
-  // global address without the plane offset, its byte offset inside a stage,
-  // its size, the plane it reads (0..3: z-1 .. z+2) and the element size;
-  // and, where the segment crosses x = 0 or x = nx (nx >= 2 BX: at most one
-  // of the two), piece B's address relative to A, stage offset and size.
-  __shared__ uint4 qdesc[2][SH::NQ];
-  for (int q = tid; q < SH::NQ; q += NT) {
-    const unsigned char* base;
-    int rsel, dz, xa, len, esz;
-    size_t dst;
+  // Copies of a stage (local plane k, plane z = zb + k): f and phi*u of the BY
+  // rows of plane z, the g of the NR phase-A rows of plane z + 1.  The BX
+  // columns of a row are 16-byte chunks that neighbouring threads copy; the
+  // chunk left or right of them, where the row's population is read there
+  // (wrapped at x = 0 and x = nx), is an item of its own.  A row and such an
+  // item are described once per CTA (only the plane changes from stage to
+  // stage): global address without the plane offset, byte offset inside a
+  // stage, and the plane it reads (0..3: z-1 .. z+2).
+  __shared__ uint4 rows[SH::NROW];
+  __shared__ uint4 pads[SH::NPAD];
+  auto desc = [&](const void* plane, int row, int x, int esz, size_t at, int dz) {
+    const uint64_t src = reinterpret_cast<uint64_t>(plane) +
+                         ((uint64_t)wrapy(y0 + row) * (uint32_t)nx + (uint32_t)x) * (uint32_t)esz;
+    return make_uint4((uint32_t)src, (uint32_t)(src >> 32), (uint32_t)at, (uint32_t)dz);
+  };
+  for (int q = tid; q < SH::NROW; q += NT) {
     if (q < 19 * BY) {  // f_i of tile row r: row y0 + r - c_iy, plane z - c_iz
-      const int i = q / BY, r = q % BY, cx = bcx(i);
-      const int lp = cx == 1 ? ES : 0, rp = cx == -1 ? ES : 0;
-      base = reinterpret_cast<const unsigned char*>(fs + (int64_t)i * P);
-      rsel = r - bcy(i), dz = 1 - bcz(i), xa = x0 - lp, len = BX + lp + rp, esz = sizeof(S);
-      dst = SH::F_OFF + (((size_t)i * BY + r) * WS + (ES - lp)) * sizeof(S);
-    } else if (q < 19 * BY + 6 * NR) {  // mover m of phase-A row r: row y0-1+r-c_my, plane z+1-c_mz
-      const int u = q - 19 * BY, m = u / NR + 1, r = u % NR, cx = bcx(m);
-      const int lp = cx == -1 ? 0 : ES, rp = cx == 1 ? 0 : ES;
-      base = reinterpret_cast<const unsigned char*>(gms + (int64_t)(m - 1) * P);
-      rsel = r - 1 - bcy(m), dz = 2 - bcz(m), xa = x0 - lp, len = BX + lp + rp, esz = sizeof(S);
-      dst = SH::GM_OFF + (((size_t)(m - 1) * NR + r) * WS + (ES - lp)) * sizeof(S);
-    } else if (q < 22 * BY + 6 * NR) {  // phi*u: row y0 + r, plane z
-      const int u = q - 19 * BY - 6 * NR, c = u / BY, r = u % BY;
-      base = reinterpret_cast<const unsigned char*>(js + (int64_t)c * P);
-      rsel = r, dz = 1, xa = x0, len = BX, esz = sizeof(T);
-      dst = SH::J_OFF + ((size_t)c * BY + r) * BX * sizeof(T);
+      const int i = q / BY, r = q % BY;
+      rows[q] = desc(fs + (int64_t)i * P, r - bcy(i), x0, sizeof(S),
+                     SH::F_OFF + (((size_t)i * BY + r) * WS + ES) * sizeof(S), 1 - bcz(i));
+    } else if (q < SH::NROW_S) {  // mover m of phase-A row r: row y0-1+r-c_my, plane z+1-c_mz
+      const int u = q - 19 * BY, m = u / NR + 1, r = u % NR;
+      rows[q] = desc(gms + (int64_t)(m - 1) * P, r - 1 - bcy(m), x0, sizeof(S),
+                     SH::GM_OFF + (((size_t)(m - 1) * NR + r) * WS + ES) * sizeof(S), 2 - bcz(m));
+    } else if (q < SH::NROW_S + 3 * BY) {  // phi*u: row y0 + r, plane z
+      const int u = q - SH::NROW_S, c = u / BY, r = u % BY;
+      rows[q] = desc(js + (int64_t)c * P, r, x0, sizeof(T),
+                     SH::J_OFF + ((size_t)c * BY + r) * BX * sizeof(T), 1);
     } else {  // g_0 (h = 0) and its low part: row y0 - 1 + r, plane z + 1
-      const int u = q - 22 * BY - 6 * NR, h = u / NR, r = u % NR;
-      base = reinterpret_cast<const unsigned char*>(h == 0 ? g0s : g0ls);
-      rsel = r - 1, dz = 2, xa = x0 - ET, len = BX + 2 * ET, esz = sizeof(T);
-      dst = SH::G0_OFF + ((size_t)h * NR + r) * WT * sizeof(T);
+      const int u = q - SH::NROW_S - 3 * BY, h = u / NR, r = u % NR;
+      rows[q] = desc(h == 0 ? g0s : g0ls, r - 1, x0, sizeof(T),
+                     SH::G0_OFF + (((size_t)h * NR + r) * WT + ET) * sizeof(T), 2);
     }
-    const unsigned char* row = base + (size_t)wrapy(y0 + rsel) * (size_t)nx * esz;
-    int xA = xa, nA = len, xB = 0, nB = 0;
-    size_t dB = 0;
-    if (xa < 0) {  // the left chunk comes from the end of the row
-      xB = nx + xa, nB = -xa, dB = dst;
-      dst += (size_t)nB * esz;
-      xA = 0, nA = len - nB;
-    } else if (xa + len > nx) {  // the right chunk comes from the start of the row
-      nA = nx - xa, nB = len - nA, xB = 0;
-      dB = dst + (size_t)nA * esz;
+  }
+  for (int q = tid; q < SH::NPAD; q += NT) {
+    if (q < 10 * BY) {  // f with c_x = 1: left, c_x = -1: right (i = 1, 7, 9, ...; 2, 8, 10, ...)
+      const int u = q / BY, r = q % BY;
+      const int i = u < 2 ? u + 1 : u + 5;
+      const bool left = bcx(i) == 1;
+      pads[q] = desc(fs + (int64_t)i * P, r - bcy(i), left ? (x0 - ES + nx) % nx : (x0 + BX) % nx,
+                     sizeof(S),
+                     SH::F_OFF + (((size_t)i * BY + r) * WS + (left ? 0 : ES + BX)) * sizeof(S),
+                     1 - bcz(i));
+    } else if (q < 10 * BY + 10 * NR) {  // movers: m = 1 left, m = 2 right, the others both
+      const int u = (q - 10 * BY) / NR, r = (q - 10 * BY) % NR;
+      const int m = u < 2 ? u + 1 : 3 + (u - 2) / 2;
+      const bool left = u < 2 ? u == 0 : (u & 1) == 0;
+      pads[q] = desc(gms + (int64_t)(m - 1) * P, r - 1 - bcy(m),
+                     left ? (x0 - ES + nx) % nx : (x0 + BX) % nx, sizeof(S),
+                     SH::GM_OFF + (((size_t)(m - 1) * NR + r) * WS + (left ? 0 : ES + BX)) * sizeof(S),
+                     2 - bcz(m));
+    } else {  // g_0 and its low part: both
+      const int u = (q - 10 * BY - 10 * NR) / NR, r = (q - 10 * BY - 10 * NR) % NR;
+      const int h = u >> 1;
+      const bool left = (u & 1) == 0;
+      pads[q] = desc(h == 0 ? g0s : g0ls, r - 1, left ? (x0 - ET + nx) % nx : (x0 + BX) % nx,
+                     sizeof(T),
+                     SH::G0_OFF + (((size_t)h * NR + r) * WT + (left ? 0 : ET + BX)) * sizeof(T), 2);
     }
-    const uint64_t srcA = reinterpret_cast<uint64_t>(row + (size_t)xA * esz);
-    qdesc[0][q] = make_uint4((uint32_t)srcA, (uint32_t)(srcA >> 32), (uint32_t)dst,
-                             (uint32_t)(nA * esz) | ((uint32_t)dz << 24) |
-                                 ((esz == 4 ? 2u : 1u) << 28));
-    qdesc[1][q] = make_uint4((uint32_t)((xB - xA) * esz), (uint32_t)dB, (uint32_t)(nB * esz), 0u);
   }
   __syncthreads();
 
-  // Issue the copies of the next stage; thread 0 first arms the stage's
-  // barrier with the stage's byte count (bytes that land before it only take
-  // the transaction count below zero for a moment; the phase cannot complete
-  // before the one arrival).  Stages are issued in order, k = 0, 1, ...:
-  // zq is the wrapped index of plane z - 1 of the next stage.
+  // Issue the copies of the next stage.  Every thread arrives once on the
+  // stage's barrier, when its own copies have landed.  Stages are issued in
+  // order, k = 0, 1, ...: zq is the wrapped index of plane z - 1 of the next.
   const uint32_t nxy = (uint32_t)nx * (uint32_t)ny;
   int zq = wrapz(zb - 1);
+  constexpr int CS = BX / ES, CT = BX / ET;  // chunks of a row's BX columns
+  static_assert(NT % CS == 0 && NT % CT == 0, "a thread keeps its chunk of the row");
   auto issue = [&](int k) {
-    unsigned char* st = stage(k);
-    uint64_t* bar = &bars[k % NST];
+    const uint32_t st = lbmk::smem_u32(stage(k));
     const int z1 = zq + 1 == nz ? 0 : zq + 1;
     const int z2 = z1 + 1 == nz ? 0 : z1 + 1;
     const int z3 = z2 + 1 == nz ? 0 : z2 + 1;
-    if (tid == 0) lbmk::mbar_arrive_expect_tx(bar, SH::TX_BYTES);
+    const uint32_t o0 = (uint32_t)zq * nxy, o1 = (uint32_t)z1 * nxy, o2 = (uint32_t)z2 * nxy,
+                   o3 = (uint32_t)z3 * nxy;
+    auto copy = [&](const uint4& d, int esz, uint32_t chunk) {
+      const uint32_t off = d.w & 2u ? (d.w & 1u ? o3 : o2) : (d.w & 1u ? o1 : o0);
+      const uint64_t src = (((uint64_t)d.y << 32) | d.x) + (uint64_t)off * (uint32_t)esz;
+      lbmk::copy16_g2s(st + d.z + chunk, src + chunk);
+    };
 #pragma unroll
-    for (int q = tid; q < SH::NQ; q += NT) {
-      const uint4 d0 = qdesc[0][q];
-      const uint32_t dz = (d0.w >> 24) & 3u;
-      const int zp = dz == 0 ? zq : (dz == 1 ? z1 : (dz == 2 ? z2 : z3));
-      const unsigned char* src =
-          reinterpret_cast<const unsigned char*>(((uint64_t)d0.y << 32) | d0.x) +
-          ((size_t)((uint32_t)zp * nxy) << (d0.w >> 28));
-      lbmk::bulk_g2s(st + d0.z, src, d0.w & 0xFFFFFFu, bar);
-      const uint4 d1 = qdesc[1][q];
-      if (d1.z) lbmk::bulk_g2s(st + d1.y, src + (int32_t)d1.x, d1.z, bar);
-    }
+    for (int q = tid; q < SH::NROW_S * CS; q += NT)
+      copy(rows[q / CS], sizeof(S), (uint32_t)(tid % CS) * 16u);
+#pragma unroll
+    for (int q = tid; q < (SH::NROW - SH::NROW_S) * CT; q += NT)
+      copy(rows[SH::NROW_S + q / CT], sizeof(T), (uint32_t)(tid % CT) * 16u);
+#pragma unroll
+    for (int q = tid; q < SH::NPAD; q += NT)
+      copy(pads[q], q < 10 * BY + 10 * NR ? (int)sizeof(S) : (int)sizeof(T), 0u);
+    lbmk::mbar_arrive_on_copies(&bars[k % NST]);
     zq = z1;
   };
 
@@ -261,7 +278,12 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
     hx = u < NR ? -1 : BX, hy = (u < NR ? u : u - NR) - 1;
   };
 
-  for (int k = 0; k < NST - 1 && k < nplanes; ++k) issue(k);
+  // a bound of 0 is tested before the prologue, which covers the copies' flight
+  bool early = false;
+  for (int k = 0; k < NST - 1 && k < nplanes; ++k) {
+    issue(k);
+    if (k == 0) early = wait_cycles <= 0 && !lbmk::mbar_test_wait(&bars[0], 0);
+  }
   int issued_last = min(NST - 1, nplanes) - 1;
   int landed = -1;
 
@@ -304,7 +326,8 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
   for (int k = 0; k < nplanes; ++k) {
     const int z = zb + k;
     unsigned char* st = stage(k);
-    const bool bad = !lbmk::mbar_wait_bounded(&bars[k % NST], (uint32_t)((k / NST) & 1), lim);
+    const bool bad = (k == 0 && early) ||
+                     !lbmk::mbar_wait_bounded(&bars[k % NST], (uint32_t)((k / NST) & 1), lim);
     if (!bad) {
       landed = k;
       // phase A of plane z + 1 from the staged g rows
@@ -337,7 +360,6 @@ __global__ void __launch_bounds__(BX* BY / 2, MINB)
     // the stage of plane k-1 is free: refill it with plane k-1+NST
     const int nxt = k + NST - 1;
     if (nxt < nplanes) {
-      lbmk::fence_proxy_async_smem();
       issue(nxt);
       issued_last = nxt;
     }

@@ -1,6 +1,6 @@
-// Inline-PTX helpers for the Blackwell bulk-copy (TMA) engine and mbarriers.
-// Only the 1-D bulk form cp.async.bulk is used: both addresses 16-byte
-// aligned, size a multiple of 16 bytes.
+// Inline-PTX helpers for the Blackwell bulk-copy (TMA) engine, per-thread
+// asynchronous copies and mbarriers.  Only the 1-D bulk form cp.async.bulk is
+// used: both addresses 16-byte aligned, size a multiple of 16 bytes.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -78,6 +78,20 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
           smem_u32(dst)),
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
+}
+
+// 16 bytes global -> shared by this thread (both addresses 16-byte aligned;
+// dst a shared-window address), past L1.
+__device__ __forceinline__ void copy16_g2s(uint32_t dst, uint64_t src) {
+  asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"(dst), "l"(src)
+               : "memory");
+}
+
+// One arrival on `bar` (counted by its initial count) when every copy16_g2s
+// this thread has issued so far has landed.
+__device__ __forceinline__ void mbar_arrive_on_copies(uint64_t* bar) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar))
+               : "memory");
 }
 
 }  // namespace lbmk
