@@ -1,17 +1,25 @@
-// TMA-staged step kernel (grids whose width nx is a multiple of 16 bytes of
-// the working type and at least 4).
+// Staged step kernel (grids whose width nx is a multiple of 16 bytes of the
+// working type and at least 4).
 //
 // Work decomposition is that of step_kernel (a CTA owns a strip of BX
 // columns and marches down `nrows` rows), but the populations reach shared
-// memory through the bulk-copy engine instead of registers: for every row
-// the CTA needs, lanes of warp 0 issue one cp.async.bulk per population plane
-// for the pulled source row (r - c_iy) over columns [x0-4, x0+wact+4) (the
-// periodic wrap in x splits a segment into at most three 16-byte aligned
-// pieces) and two for phi*u of the previous step.  Completion is tracked by
-// one mbarrier per stage with its transaction byte count.  S stages form a
-// ring; rows are fetched S-1 ahead of the collision, so the consumer threads
-// never wait on DRAM latency.  The halo columns of the phi/psi ring come from
-// the same staged segments, without extra global loads.
+// memory by asynchronous 16-byte copies instead of registers: for every row
+// the CTA needs, its threads copy the pulled source rows (r - c_iy) of every
+// population plane over columns [x0, x0+wact), the chunks beside them that the
+// pull reads (periodic in x), and phi*u of the previous step.  Completion is
+// counted on one mbarrier per stage.  S stages form a ring; rows are fetched
+// S-1 ahead of the collision, so the consumer threads seldom wait on DRAM
+// latency.  The halo columns of the phi/psi ring come from the same staged
+// rows, without extra global loads.
+//
+// Why threads copy and not the bulk engine: a bulk copy takes its operands
+// from uniform registers, so the 20 and more rows of a stage (512 bytes each)
+// were issued lane after lane by one warp, for which the others waited.  A
+// thread's 5 or 6 chunk copies are spread over the CTA.  FP32, 512 uneven cases
+// with per-step volumes, 32 steps 41.6 -> 38.5 ms; 8192 x 4096 grid, 32 steps
+// 31.7 -> 30.0 ms.  FP64 is bound by its pipe (18.4 ms either way for 64 uneven
+// cases).  What bounds it now: HBM (0.87 of the measured copy rate on the
+// large grid, the state's read-out included).
 //
 // Every wait of the consumers is bounded (StepArgs::wait_cycles); on expiry
 // the CTA raises kFlagTimeout, waits for its own copies still in flight
@@ -42,6 +50,7 @@ struct TmaShape {
   static constexpr int NPL = COUPLED ? 18 : 9;        // population planes
   static constexpr int NJ = (MODE == kModeStep) ? 2 : 0;  // phi*u planes
   static constexpr int STAGE = NPL * SEG + NJ * BX;   // elements per stage
+  static constexpr int NPAD_G = 12, NPAD = COUPLED ? 18 : 12;  // chunks beside the strip: g, all
   static constexpr size_t STAGE_BYTES = (size_t)STAGE * sizeof(T);
   static constexpr size_t BAR_OFF = S * STAGE_BYTES;
   static constexpr size_t RING_OFF = (BAR_OFF + S * 8 + 127) / 128 * 128;
@@ -55,7 +64,7 @@ struct TmaShape {
 // nx <= BX) or not; the kernel picks one per CTA, so that the strips of wide
 // rows keep compile-time staged positions.
 template <typename T, int BX, bool COUPLED, int MODE, int S, bool FROW>
-__device__ __forceinline__ void tma_body(const StepArgs<T>& a) {
+__device__ __forceinline__ void tma_body(const StepArgs<T>& a, uint4* const rows) {
   using SH = TmaShape<T, BX, COUPLED, MODE, S>;
   constexpr int SEG = SH::SEG, NPL = SH::NPL, NJ = SH::NJ, STAGE = SH::STAGE;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -115,81 +124,76 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a) {
   auto parity_of = [](int k) -> uint32_t { return (uint32_t)(((k + 1) / S) & 1); };
   auto stage_of = [&](int k) -> T* { return stages + slot_of(k) * STAGE; };
 
+  // What a row copies, described once per CTA: the planes' own columns (g 0-8,
+  // f 9-17, phi*u), and the chunks left and right of them that the pull reads
+  // (wrapped at x = 0 and x = nx): left the g planes with c_x >= 0 (the halo
+  // column -1 pulls from -1 - c_x) and the f planes with c_x = +1 (column 0
+  // pulls from -1), right the mirror image.  {plane address, element offset in
+  // a stage, column and which of rows r, r-1, r+1}.
+  constexpr int E = 16 / (int)sizeof(T);  // elements of a chunk
+  constexpr int CC = BX / E;              // chunks of a strip's columns
+  constexpr int NPAD_G = SH::NPAD_G, NPAD = SH::NPAD;
+  auto desc = [&](const T* plane, int at, int x, int cy) {
+    const uint64_t p = reinterpret_cast<uint64_t>(plane);
+    return make_uint4((uint32_t)p, (uint32_t)(p >> 32), (uint32_t)at,
+                      ((uint32_t)x << 2) | (cy == 0 ? 0u : (cy == 1 ? 1u : 2u)));
+  };
+  if (tid < NPL + NJ) {
+    const int i = tid < 9 ? tid : tid - 9;
+    rows[tid] = tid < NPL ? desc((tid < 9 ? gs : fs) + (size_t)i * P, tid * SEG + 4, x0, cy_of(i))
+                          : desc(Js + (size_t)(tid - NPL) * P, NPL * SEG + (tid - NPL) * BX, x0, 0);
+  }
+  for (int q = tid; q < NPAD; q += BX) {
+    // planes, four bits each: g left 0 1 2 4 5 8, right 0 2 3 4 6 7; f left 1 5 8, right 3 6 7
+    const bool g = q < NPAD_G, left = g ? q < 6 : q < NPAD_G + 3;
+    const int u = g ? (left ? q : q - 6) : (left ? q - NPAD_G : q - NPAD_G - 3);
+    const int i = (int)(((g ? (left ? 0x854210u : 0x764320u) : (left ? 0x851u : 0x763u)) >> (4 * u)) & 15u);
+    const int x = left ? (x0 == 0 ? nx : x0) - E : (x0 + wact >= nx ? 0 : x0 + wact);
+    rows[NPL + NJ + q] = desc((g ? gs : fs) + (size_t)i * P,
+                              (g ? i : 9 + i) * SEG + (left ? 4 - E : 4 + wact), x, cy_of(i));
+  }
   if (tid == 0) {
-    for (int s = 0; s < S; ++s) mbar_init(&bars[s], 1);
+    for (int s = 0; s < S; ++s) mbar_init(&bars[s], BX);
     fence_mbar_init();
   }
   __syncthreads();
 
-  // Issue the bulk copies of local row k (k in [-1, nrows]); warp 0 only.
-  // Rows -1 and nrows (the halo rows of the item) need the g planes only.
+  // Issue the copies of local row k (k in [-1, nrows]): 16-byte chunks, one
+  // per thread and pass, a thread keeping its chunk of the strip.  Rows -1 and
+  // nrows (the halo rows of the item) need the g planes only.  Every thread
+  // arrives once on the stage's barrier, when its own copies have landed.
   auto issue = [&](int k) {
     const bool full = (k >= 0 && k < nrows);
-    const int np = full ? NPL : 9;
-    const int nj = full ? NJ : 0;
-    T* st = stage_of(k);
-    uint64_t* bar = &bars[slot_of(k)];
-    // Staged column j holds global column (x0 - 4 + j) mod nx, j < wact + 8.
-    // Where the strip touches the periodic edge of the row, the four columns
-    // beyond it come from the other end of the row in a separate 16-byte
-    // copy, made only for the planes that read them: on the left (x0 = 0)
-    // the g planes with c_x >= 0 (the halo column -1 pulls from -1 - c_x)
-    // and the f planes with c_x = +1 (column 0 pulls from -1); on the right
-    // the mirror image.  That is 6 g and 3 f planes a side instead of 18.
-    // Lane l copies plane l (g planes 0-8, then f planes 9-17); bit l of
-    // kNeedL / kNeedR says whether it needs the left / right wrap columns.
-    constexpr uint32_t kNeedL = 0x137u | (0x122u << 9);  // g: c_x >= 0; f: c_x = +1
-    constexpr uint32_t kNeedR = 0x0DDu | (0x0C8u << 9);  // g: c_x <= 0; f: c_x = -1
-    const bool lw = (x0 == 0), rw = (x0 + wact >= nx);
-    uint32_t elems = (uint32_t)(np * (wact + 8) + nj * wact);
-    if (frow) {  // one copy of the whole row per plane
-      elems = (uint32_t)(np * nx + nj * wact);
-    } else if (lw || rw) {  // the wrap columns that no plane reads are not copied
-      const int nwrap = (full && COUPLED) ? 9 : 6;  // 6 g planes, + 3 f planes on full rows
-      elems -= (uint32_t)((lw ? 4 * (np - nwrap) : 0) + (rw ? 4 * (np - nwrap) : 0));
-    }
-    if (lane == 0) mbar_arrive_expect_tx(bar, elems * (uint32_t)sizeof(T));
-    __syncwarp();
+    T* const st = stage_of(k);
+    const uint32_t st32 = smem_u32(st);
     const int r = wrap(y0 + k);
     const uint32_t nn = (uint32_t)nx * (uint32_t)ny;
-    // one bulk copy of n elements from position `first` of a plane (checked
-    // build: the source range must lie in the plane's nodes and the target
+    const uint32_t r0 = (uint32_t)r * (uint32_t)nx, rm = (uint32_t)wrap(r - 1) * (uint32_t)nx,
+                   rp = (uint32_t)wrap(r + 1) * (uint32_t)nx;  // pull: source row r - c_iy
+    // (checked build: the source must lie in the plane's nodes and the target
     // in this stage; otherwise the copy is redirected, see lbm_check.h)
-    auto copy = [&](T* dst, const T* plane, const T* buf, int64_t first, uint32_t n) {
-      const bool ok = LBM_BOUND(a.flags, first, nn) && LBM_BOUND(a.flags, first + n - 1, nn) &&
-                      LBM_BOUND(a.flags, (dst - st) + n - 1, STAGE);
-      bulk_g2s(ok ? dst : st, ok ? plane + first : buf, n * sizeof(T), bar);
+    auto copy = [&](const uint4 d, uint32_t c) {
+      const uint32_t code = d.w & 3u;
+      const uint32_t first = (code == 0 ? r0 : (code == 1 ? rm : rp)) + (d.w >> 2) + c;
+      const uint64_t plane = ((uint64_t)d.y << 32) | d.x;
+      const bool ok = LBM_BOUND(a.flags, first + (E - 1), nn) &&
+                      LBM_BOUND(a.flags, d.z + c + (E - 1), STAGE);
+      copy16_g2s(st32 + (ok ? (d.z + c) * (uint32_t)sizeof(T) : 0u),
+                 ok ? plane + (uint64_t)first * sizeof(T) : plane);
     };
-    if (lane < np) {
-      const int i = lane < 9 ? lane : lane - 9;
-      const T* buf = lane < 9 ? gs : fs;
-      const T* plane = buf + (size_t)i * P;
-      const int64_t row = (int64_t)wrap(r - cy_of(i)) * nx;  // pull: source row r - c_iy
-      T* dst = st + lane * SEG;
-      int j = 0, g0, len;
-      if (frow) {
-        copy(dst + 4, plane, buf, row, (uint32_t)nx);
-      } else {
-        if (lw) {
-          if ((kNeedL >> lane) & 1u) copy(dst, plane, buf, row + (nx - 4), 4);
-          j = 4;
-          g0 = 0;
-          len = wact;
-        } else {
-          g0 = x0 - 4;
-          len = wact + 4;
-        }
-        if (!rw) {
-          copy(dst + j, plane, buf, row + g0, (uint32_t)(len + 4));
-        } else {
-          copy(dst + j, plane, buf, row + g0, (uint32_t)len);
-          if ((kNeedR >> lane) & 1u) copy(dst + j + len, plane, buf, row, 4);
-        }
+    const int np = full ? NPL + NJ : 9;
+    const uint32_t c = (uint32_t)(tid % CC) * E;
+    if ((int)c < wact) {
+#pragma unroll
+      for (int it = 0; it < (NPL + NJ + E - 1) / E; ++it) {
+        const int p = tid / CC + it * E;
+        if (p < np) copy(rows[p], c);
       }
-    } else if (lane >= NPL && lane < NPL + nj) {
-      const int q = lane - NPL;
-      copy(st + NPL * SEG + q * BX, Js + (size_t)q * P, Js, (int64_t)r * nx + x0, (uint32_t)wact);
     }
+    if (!frow) {  // a whole row has its neighbours in its own copy
+      for (int q = tid; q < (full ? NPAD : NPAD_G); q += BX) copy(rows[NPL + NJ + q], 0u);
+    }
+    mbar_arrive_on_copies(&bars[slot_of(k)]);
   };
 
   // g of a local column from a staged row, given the staged positions of
@@ -218,14 +222,15 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a) {
   };
 
   // ---- prologue: rows -1 .. S-2 in flight; phi of rows -1 and 0 ----------
-  if (warp == 0) {
-    const int last = min(S - 2, nrows);
-    for (int k = -1; k <= last; ++k) issue(k);
+  const long long lim = a.wait_cycles;
+  bool early = false;  // a bound of 0 is tested before the later rows' issue covers the flight
+  for (int k = -1; k <= min(S - 2, nrows); ++k) {
+    issue(k);
+    if (k == -1) early = lim <= 0 && !mbar_test_wait(&bars[slot_of(-1)], parity_of(-1));
   }
   // rows up to `landed` have been seen complete by this thread
   int landed = -2;
-  const long long lim = a.wait_cycles;
-  bool bad = !mbar_wait_bounded(&bars[slot_of(-1)], parity_of(-1), lim);
+  bool bad = early || !mbar_wait_bounded(&bars[slot_of(-1)], parity_of(-1), lim);
   if (!bad) {
     landed = -1;
     put_row(-1);
@@ -264,10 +269,7 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a) {
     // the stage of row k-1 is free: refill it with row k-1+S
     const int nxt = k - 1 + S;
     if (nxt <= nrows) {
-      if (warp == 0) {
-        fence_proxy_async_smem();
-        issue(nxt);
-      }
+      issue(nxt);
       issued_last = nxt;
     }
     if (act) {
@@ -332,11 +334,13 @@ constexpr int tma_min_blocks() {
 template <typename T, int BX, bool COUPLED, int MODE, int S>
 __global__ void __launch_bounds__(BX, (tma_min_blocks<T, BX>()))
     step_kernel_tma(const StepArgs<T> a) {
+  using SH = TmaShape<T, BX, COUPLED, MODE, S>;
+  __shared__ uint4 rows[SH::NPL + SH::NJ + SH::NPAD];
   const Item it = a.items[blockIdx.x];
   if (it.x0 == 0 && a.cases[it.c].nx <= BX)
-    tma_body<T, BX, COUPLED, MODE, S, true>(a);
+    tma_body<T, BX, COUPLED, MODE, S, true>(a, rows);
   else
-    tma_body<T, BX, COUPLED, MODE, S, false>(a);
+    tma_body<T, BX, COUPLED, MODE, S, false>(a, rows);
 }
 
 }  // namespace lbmk
