@@ -77,14 +77,23 @@ class AdjointSim:
     def t(self):
         return lbm.lbm_time(self.h)
 
+    def _after_current(self):
+        """Orders the handle's stream after the caller's: a new buffer may be memory
+        that the caller's stream still works on."""
+        cur = torch.cuda.current_stream(self.dev)
+        if cur != self.sim.stream:
+            self.sim.stream.wait_stream(cur)
+
     def phi(self):
         out = torch.empty(self.shape, dtype=torch.float64, device=self.dev)
+        self._after_current()
         lbm.lbm_field_phi(self.h, 0, out.data_ptr())
         return out
 
     def seed_phi(self, dphi):
         adj = torch.empty((20,) + self.shape, dtype=self.dtype, device=self.dev)
         dphi = dphi.to(device=self.dev, dtype=torch.float64).contiguous()
+        self._after_current()
         lbm.lbm_adjoint_seed_phi(self.h, dphi.data_ptr(), adj.data_ptr())
         return adj
 
