@@ -249,10 +249,24 @@ template <>
 cudaError_t launch_snapshot<LBM_T>(const LBM_T* f, const LBM_T* g, const LBM_T* J,
                                    const LBM_T* lo, int64_t P, int64_t n, LBM_T* out,
                                    cudaStream_t s) {
-  const int planes = lo ? 21 : 20;
-  const dim3 grid((unsigned)std::min<int64_t>((n + 255) / 256, 4096), planes);
-  snapshot_kernel<LBM_T><<<grid, 256, 0, s>>>(f, g, J, lo, P, n, out);
-  return cudaGetLastError();
+  constexpr int E = 16 / (int)sizeof(LBM_T);
+  // plane strides and buffers of the handle are multiples of 16 bytes
+  const bool vec = n % E == 0 && (uintptr_t)out % 16 == 0 && P % E == 0;
+  const int64_t m = vec ? n / E : n;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)std::min<int64_t>((m + 511) / 512, 4096), lo ? 21 : 20);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  // (not into a graph, where the kernel before it may be several)
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+  cfg.numAttrs = st == cudaStreamCaptureStatusNone ? 1 : 0;
+  return vec ? cudaLaunchKernelEx(&cfg, snapshot_kernel<LBM_T, uint4>, f, g, J, lo, P, n, out)
+             : cudaLaunchKernelEx(&cfg, snapshot_kernel<LBM_T, LBM_T>, f, g, J, lo, P, n, out);
 }
 
 template <>

@@ -167,7 +167,7 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a, uint4* const rows
     T* const st = stage_of(k);
     const uint32_t st32 = smem_u32(st);
     const int r = wrap(y0 + k);
-    const uint32_t nn = (uint32_t)nx * (uint32_t)ny;
+    [[maybe_unused]] const uint32_t nn = (uint32_t)nx * (uint32_t)ny;
     const uint32_t r0 = (uint32_t)r * (uint32_t)nx, rm = (uint32_t)wrap(r - 1) * (uint32_t)nx,
                    rp = (uint32_t)wrap(r + 1) * (uint32_t)nx;  // pull: source row r - c_iy
     // (checked build: the source must lie in the plane's nodes and the target
