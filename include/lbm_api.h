@@ -262,7 +262,7 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel,
                  int32_t* best_bx, int32_t* best_rows, double* best_ms);
 
 /* Step-kernel variant: 0 = automatic, 1 = register-pipelined loads (any
- * grid), 2 = bulk-copy (TMA) staged loads through shared memory (needs every
+ * grid), 2 = loads staged through shared memory by asynchronous copies (needs every
  * case to have nx >= 4 and nx a multiple of 4 in FP32, of 2 in FP64), 3 = one
  * cooperative launch for many steps (at most 4 Mi nodes; the chip-resident
  * kernel where the batch fits it, see lbm_step, else a grid barrier between
