@@ -60,7 +60,7 @@ def parse():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-extras", action="store_true")
     ap.add_argument("--cpu-seconds", type=float, default=15.0)
-    ap.add_argument("--kernel", type=int, default=0, help="0 auto, 1 register, 2 bulk-copy")
+    ap.add_argument("--kernel", type=int, default=0, help="0 auto, 1 register, 2 staged")
     ap.add_argument("--tiling", type=str, default=None, help="BX,ROWS (default: autotuned)")
     ap.add_argument("--no-autotune", action="store_true")
     ap.add_argument("--chains", type=int, default=0,

@@ -174,7 +174,7 @@ int lbm_set_chains(lbm_handle* h, int32_t nchains);
 int32_t lbm_get_chains(const lbm_handle* h);
 
 /* Whole-row chains (on = 1; off by default; lbm_autotune tries both): with
- * the bulk-copy kernel in FP32 and strips of 128 columns, a case whose row
+ * the staged kernel in FP32 and strips of 128 columns, a case whose row
  * fits a width of 64, 96, 192 or 256 columns (the smallest that holds it,
  * 128 included, decides) runs each row as one strip of that width, in one
  * extra chain per width.  A whole-row strip copies its row once per plane and
@@ -188,7 +188,7 @@ int32_t lbm_get_chains(const lbm_handle* h);
 int lbm_set_row_chains(lbm_handle* h, int32_t on);
 int32_t lbm_get_row_chains(const lbm_handle* h);
 
-/* Bound of the device waits, in SM clock cycles: the bulk-copy kernel's
+/* Bound of the device waits, in SM clock cycles: the staged kernel's
  * waits for its staged rows, the chip-resident kernel's waits for its
  * neighbours' rims and the persistent kernel's grid barrier.  A
  * wait that gives up raises LBM_ERR_TIMEOUT (reported by the next
@@ -270,7 +270,7 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel,
  * lbm_set_tiling).  lbm_get_kernel returns the variant of single steps in use
  * (1 or 2, or 3 if asked for).
  * Changing the variant rebuilds the work-item table (whole-row chains run
- * the bulk-copy kernel only; synchronises). */
+ * the staged kernel only; synchronises). */
 int lbm_set_kernel(lbm_handle* h, int32_t variant);
 int32_t lbm_get_kernel(const lbm_handle* h);
 

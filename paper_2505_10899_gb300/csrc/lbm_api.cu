@@ -837,7 +837,7 @@ size_t state_bytes_case(const lbm_handle* h, int k) {
 }
 
 // New tiling or chain count: rebuild the item table and the case table.
-// Whole-row chains need the bulk-copy kernel (FP32; the FP64 kernels are
+// Whole-row chains need the staged kernel (FP32; the FP64 kernels are
 // bound by the FP64 pipe, where the strip layout hardly matters).
 bool rowmode(const lbm_handle* h) {
   return h->row_chains && use_tma(h) && h->precision == LBM_F32;
@@ -961,7 +961,7 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t 
     h->tma_ok = true;
     for (int k = 0; k < ncases; ++k)
       if (cases[k].nx % vec != 0 || cases[k].nx < 4) h->tma_ok = false;
-    // the bulk-copy kernel stages periodic source rows only: walls run the
+    // the staged kernel stages periodic source rows only: walls run the
     // register-pipelined kernel
     for (int k = 0; k < ncases; ++k)
       if (cases[k].walls) h->tma_ok = false;
@@ -985,7 +985,7 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t 
     if (cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming) != cudaSuccess)
       return cleanup(fail(LBM_ERR_CUDA, "cannot create chain events"));
   }
-  if (h->tma_ok) {  // handles without the bulk-copy kernel need no attributes of it
+  if (h->tma_ok) {  // handles without the staged kernel need no attributes of it
     cudaError_t e = h->precision == LBM_F32 ? lbmk::prepare_tma<float>() : lbmk::prepare_tma<double>();
     if (e != cudaSuccess)
       return cleanup(fail(LBM_ERR_CUDA, std::string("kernel attributes: ") + cudaGetErrorString(e)));
@@ -1238,7 +1238,7 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
     if (kv == 3 && total_nodes(h) > kPersistMaxNodes) continue;
     for (int bx : {128, 64, 32}) {
       for (int rows : {2, 4, 8, 16, 32, 64, 128}) {
-        // whole-row chains exist for the FP32 bulk-copy kernel on 128-wide
+        // whole-row chains exist for the FP32 staged kernel on 128-wide
         // strips only: try them on and off there
         const int nrc = (kv == 2 && bx == 128 && h->precision == LBM_F32) ? 2 : 1;
         for (int rcv = 0; rcv < nrc; ++rcv) {
