@@ -342,7 +342,11 @@ int lbm_record_steps(lbm_handle* h, int64_t count, void* d_states, int64_t strid
  * the high part of its float pair, a difference of at most half an FP32 ulp
  * of g_0 in phi).
  *   lbm_adjoint_attach: device scratch of lbm_adjoint_workspace_bytes()
- *     bytes (256-byte aligned, caller-owned, outlives the handle).
+ *     bytes (256-byte aligned, caller-owned, outlives the handle).  From here
+ *     on an FP64 handle steps by division, root, logarithm and the general
+ *     collision in place of their short forms, and takes the chip-resident
+ *     kernel only where that gives the bits of its single steps: derivatives
+ *     through psi (slope up to 1/xi) move by up to 1e-8 with a state's last bit.
  *   lbm_adjoint_seed_phi: adjoint state of an objective that depends on the
  *     current phi only, from its FP64 field derivative d_dphi [ny][nx]
  *     (phi = sum of the pulled g, Eq. 35).

@@ -36,6 +36,7 @@
 
 namespace lbmk {
 int set_last_error(int code, const char* msg);
+void drop_graphs(lbm_handle* h);
 }  // namespace lbmk
 
 using lbmk::CaseDev;
@@ -165,8 +166,6 @@ struct AdArgs {
 // which the normal of Eq. 17 does not see).
 template <typename R>
 __device__ __forceinline__ R dpsi_dphi(R p, R xi) {
-  if constexpr (sizeof(R) == 8)
-    return lbmk::rcp64(p + xi) + lbmk::rcp64((R(1) - p) + xi);
   const R d = R(1) / (p + xi) + R(1) / ((R(1) - p) + xi);
   return sizeof(R) == 4 ? R(1.4426950408889634) * d : d;
 }
@@ -904,6 +903,11 @@ int lbm_adjoint_attach(lbm_handle* h, void* d_scratch, size_t bytes) {
   h->adj_ws_bytes = bytes;
   h->adj_res = lbmk::res_plan_adjoint(h->params[0]);
   h->adj_epoch = 1;
+  if (h->precision == LBM_F64 && !h->pd.plain) {  // see Phys::plain
+    lbmk::drop_graphs(h);                         // captured launches hold the short forms
+    h->pd.plain = 1;
+    h->pd.unit = 0;
+  }
   const AdScratch s = carve(h);
   cudaError_t e = cudaMemsetAsync(s.part, 0, (kAdBlocks + 1) * kNParam * sizeof(double),
                                   h->stream);  // partials and accumulator

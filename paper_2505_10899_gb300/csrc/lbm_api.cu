@@ -472,12 +472,21 @@ int launch_persist(lbm_handle* h, cudaStream_t s, int parity, int nsteps, int fl
   return LBM_OK;
 }
 
+// Whether the chip-resident kernel may run this handle's steps at all.  A
+// handle with reverse mode in FP64 (Phys::plain) takes it only where the
+// single steps run the staged kernel, whose bits it gives; the register
+// kernel contracts some multiply-adds differently, and the parameter
+// derivatives of a state that differs in its last bits differ by 1e-9.
+bool res_allowed(const lbm_handle* h) {
+  return h->res.variant >= 0 && (!h->pd.plain || h->tma_ok);
+}
+
 // Whether a run of nsteps steps takes the chip-resident kernel: the batch
 // fits, no other kernel was asked for, no per-step volumes are tracked, and
 // the stream is not being captured (a replayed launch would reuse its tags).
 constexpr int64_t kResMinSteps = 4;
 bool use_resident(const lbm_handle* h, int64_t nsteps) {
-  if (h->res.variant < 0 || h->track || (h->kernel != 0 && h->kernel != 3) ||
+  if (!res_allowed(h) || h->track || (h->kernel != 0 && h->kernel != 3) ||
       nsteps < (h->kernel == 3 ? 1 : kResMinSteps))
     return false;
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
@@ -881,6 +890,7 @@ int retile(lbm_handle* h, const Tiling& t, int nchains) {
 
 namespace lbmk {
 int set_last_error(int code, const char* msg) { return fail(code, msg); }
+void drop_graphs(lbm_handle* h) { drop_graph(h); }
 }  // namespace lbmk
 
 // ============================================================================
@@ -1248,7 +1258,7 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
           if (rc != LBM_OK) break;
           int n_run = n_trial;
           cudaError_t e = cudaSuccess;
-          if (kv == 3 && h->res.variant >= 0) {
+          if (kv == 3 && res_allowed(h)) {
             // the chip-resident kernel has tiles of its own: one trial
             if (bx != 128 || rows != 2) continue;
             n_run = std::max(n_trial, kGraphSteps);
@@ -1288,7 +1298,7 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
             best = ms / n_run;
             best_t.bx = bx;
             best_t.rows = rows;
-            if (kv == 3 && h->res.variant >= 0) best_t = keep_tile;
+            if (kv == 3 && res_allowed(h)) best_t = keep_tile;
             best_k = kv;
             best_rc = rcv == 1;
           }

@@ -171,7 +171,6 @@ __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T
   const int hcm = (hc == 0) ? nx - 1 : hc - 1;
   const int hcp = (hc == nx - 1) ? 0 : hc + 1;
 
-  const T xi = a.ph.xi;
   const bool do_vol = (MODE == kModeStep) && (a.vol_part != nullptr);
   double vacc = 0.0;
   CaseK<T> K = case_consts<T, COUPLED>(a, cdp, xc);
@@ -243,11 +242,11 @@ __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T
     const int s = (k + 4) & 3;
     if (act) {
       const T phi = sum9(G);
-      ring.put(s, tid + 1, phi, psi_of(phi, xi));
+      ring.put(s, tid + 1, phi, psi_of(phi, a.ph));
     }
     if (hthr) {
       const T phi = sum9(H);
-      ring.put(s, hslot, phi, psi_of(phi, xi));
+      ring.put(s, hslot, phi, psi_of(phi, a.ph));
     }
   };
 

@@ -114,7 +114,6 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a, uint4* const rows
   const int om = spos(tid, -1), o0 = spos(tid, 0), op = spos(tid, 1);
   const int hm = spos(hcol, -1), h0 = spos(hcol, 0), hp = spos(hcol, 1);
 
-  const T xi = a.ph.xi;
   const bool do_vol = (MODE == kModeStep) && (a.vol_part != nullptr);
   double vacc = 0.0;
   CaseK<T> K = case_consts<T, COUPLED>(a, cdp, xc);
@@ -212,12 +211,12 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a, uint4* const rows
     if (act) {
       staged_g(st, om, o0, op, G);
       const T phi = sum9(G);
-      ring.put(s, tid + 1, phi, psi_of(phi, xi));
+      ring.put(s, tid + 1, phi, psi_of(phi, a.ph));
     }
     if (hthr) {
       staged_g(st, hm, h0, hp, G);
       const T phi = sum9(G);
-      ring.put(s, hslot, phi, psi_of(phi, xi));
+      ring.put(s, hslot, phi, psi_of(phi, a.ph));
     }
   };
 

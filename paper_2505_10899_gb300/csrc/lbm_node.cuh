@@ -38,10 +38,10 @@ struct Num<float> {
 
 template <>
 struct Num<double> {
-  static __device__ __forceinline__ double rsq(double x) { return rsq64(x); }
-  static __device__ __forceinline__ double rcp(double x) { return rcp64(x); }
+  static __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
+  static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
   static __device__ __forceinline__ double lratio(double a, double b) {
-    return lratio64(a, b);
+    return log(a / b);
   }
   static __device__ __forceinline__ double clamp01(double v) {
     return fmin(fmax(v, 0.0), 1.0);
@@ -84,6 +84,30 @@ template <typename T>
 __device__ __forceinline__ T psi_of(T phi, T xi) {
   const T pc = Num<T>::clamp01(phi);
   return Num<T>::lratio(pc + xi, (T(1) - pc) + xi);
+}
+
+// The same, a reciprocal and a reciprocal square root in the forward step: in
+// FP64 the short forms of lbm_math.cuh, unless the handle asks for the division,
+// root and logarithm of Num<double> (Phys::plain, a launch-uniform branch: 64
+// uneven FP64 cases, 8 steps 18.16 ms without it, 17.90 with it).
+template <typename T>
+__device__ __forceinline__ T psi_of(T phi, const Phys<T>& ph) {
+  if constexpr (sizeof(T) == 8) {
+    const T pc = Num<T>::clamp01(phi), a = pc + ph.xi, b = (T(1) - pc) + ph.xi;
+    return ph.plain ? Num<T>::lratio(a, b) : lratio64(a, b);
+  } else {
+    return psi_of(phi, ph.xi);
+  }
+}
+template <typename T>
+__device__ __forceinline__ T step_rcp(T x, const Phys<T>& ph) {
+  if constexpr (sizeof(T) == 8) return ph.plain ? Num<T>::rcp(x) : rcp64(x);
+  else return Num<T>::rcp(x);
+}
+template <typename T>
+__device__ __forceinline__ T step_rsq(T x, const Phys<T>& ph) {
+  if constexpr (sizeof(T) == 8) return ph.plain ? Num<T>::rsq(x) : rsq64(x);
+  else return Num<T>::rsq(x);
 }
 
 // Forward moments m = M v (rows of Eq. 24) by butterflies.
@@ -269,7 +293,7 @@ __device__ __forceinline__ void f_unit(const CaseK<double>& K, double (&F)[9], d
   if (MODE != kModeStep) return;
   double sD7 = K.sD7, hD7 = K.hD7;
   if (K.var_tau) {
-    const double s7 = Num<double>::rcp(3.0 * (K.mu_g + phi * K.dmu) * irho + 0.5);  // Eq. 27
+    const double s7 = rcp64(3.0 * (K.mu_g + phi * K.dmu) * irho + 0.5);  // Eq. 27
     sD7 = -0.25 * s7;
     hD7 = 0.25 - 0.125 * s7;
   }
@@ -343,7 +367,7 @@ __device__ __forceinline__ NodeOut<T> node_update(const Phys<T>& ph, const CaseK
   bool unit = false;  // FP64 with unit free rates: the short collision
   if (COUPLED) {
     const T rho = K.rho_g + phi * K.drho;  // linear rho(phi)
-    const T irho = Num<T>::rcp(rho);
+    const T irho = step_rcp(rho, ph);
     if constexpr (sizeof(T) == 8) {
       if (ph.unit) {
         f_unit<MODE>(K, Fc, phi, rho, irho, gpx, gpy, Fx, Fy, o);
@@ -375,7 +399,7 @@ __device__ __forceinline__ NodeOut<T> node_update(const Phys<T>& ph, const CaseK
       if (K.var_tau) {
         const T mu_v = K.mu_g + phi * K.dmu;
         const T tau = T(3) * mu_v * irho + T(0.5);  // Eq. 27
-        const T s7 = Num<T>::rcp(tau);
+        const T s7 = step_rcp(tau, ph);
         sD7 = T(-0.25) * s7;
         hD7 = T(0.25) - T(0.125) * s7;
       }
@@ -406,7 +430,7 @@ __device__ __forceinline__ NodeOut<T> node_update(const Phys<T>& ph, const CaseK
     const T pc = Num<T>::clamp01(phi);
     const T ta = pc + ph.xi, tb = (T(1) - pc) + ph.xi;
     const T q2 = qx * qx + qy * qy;
-    const T iq = (q2 >= ph.qmin2) ? Num<T>::rsq(q2) : T(0);  // n := 0 on ridges of psi
+    const T iq = (q2 >= ph.qmin2) ? step_rsq(q2, ph) : T(0);  // n := 0 on ridges of psi
     // (lambda/W) [1 - tanh^2(2psi/W)] / |grad psi|, tanh via Eqs. 13-15
     const T sh = ph.lamW * ph.tfac * ta * tb * iq;
     const T Vx = T(3) * dJx + sh * qx;  // d_t(phi u)/c_s^2 + sharpening flux

@@ -153,7 +153,6 @@ __global__ void __launch_bounds__(NT, MINB)
   const uint32_t P = (uint32_t)cdp->plane, nn = (uint32_t)nx * (uint32_t)ny;
   const bool walls = cdp->walls != 0;
   const bool wbot = walls && tl.y0 == 0, wtop = walls && tl.y0 + h == ny;
-  const T xi = a.ph.xi;
   auto cell_of = [&](int x, int y) -> int { return (y + 2) * pw + x + 2; };
 
   const T* gs = cdp->g[a.parity];
@@ -347,7 +346,7 @@ __global__ void __launch_bounds__(NT, MINB)
     const T phi = sum9(G);
     typename Pair<T>::type v;
     v.x = phi;
-    v.y = psi_of(phi, xi);
+    v.y = psi_of(phi, a.ph);
     pq[dst] = v;
   };
   // own nodes away from the tile's edge: no rim needed
