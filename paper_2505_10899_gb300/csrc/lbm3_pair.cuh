@@ -4,15 +4,29 @@
 // issue in FP16 storage, so it costs what its instructions count.
 //
 // The same equations as node3, in fewer operations:
-//   - a pair (c, -c) of f: f*_{+-} = (1 - w_f) f + s +- v, with
+//   - a pair (c, -c) of f: f*_{+-} = f + (s - w_f S/2) +- (v - w_f D/2), with
+//       S, D the pair's sum and difference,
 //       s = w w_f base + (c.u) [4.5 w w_f rho (c.u) + 3 w h_f (c.grad rho)],
 //       v = c.[3 w (w_f rho u + h_f F)],
 //     the bracketed vectors formed once per weight;
 //   - the stencil's column sums and differences serve both nodes, phi and psi
 //     packed.
-// (1 - w_f) + w_f has to be 1 exactly: a rounded complement would scale the
-// conserved moments by its error at every step.  So w_f is taken back from the
-// complement (exact: both lie in [0, 2], Sterbenz).
+// What a node conserves must not be scaled by a constant that is off by a
+// rounding: every step would scale it again (rho u by 3e-8 w_f a step with the
+// FP32 1/6, 1e-5 after 200 steps).  So base and w_f rho u + h_f F, which differ
+// from node to node and so round either way, are divided by 18 and 6 with the
+// constants' low parts; and f takes the small change of a collision, with one
+// rounding at its own size and w_f unrounded at any relaxation time (a complement
+// 1 - w_f loses a bit of it per doubling of tau_f above 2).
+// Error against 64 bits, mean of 24 boxes of 64 x 40 x 40, FP32, register kernel /
+// complement and rounded constants / this form:
+//   column, tau_f 0.6: phi 4.96e-8 / 4.91e-8 / 4.87e-8, u 4.0e-6 / 7.5e-6 / 9.3e-7,
+//                      p 1.9e-6 / 2.9e-6 / 3.4e-7
+//   ball, tau_f 1:     phi 3.4e-7 / 2.9e-7 / 6.4e-8, u 2.7e-6 / 2.6e-6 / 3.5e-7,
+//                      p 8.1e-6 / 1.0e-5 / 6.7e-6
+//   ball, tau_f 9.3:   phi 6.4e-8 / 6.3e-8 / 4.9e-8, u 3.0e-7 / 2.5e-7 / 7.0e-8,
+//                      p 6.3e-6 / 5.7e-6 / 5.0e-6
+// It costs 1.8% in FP16 storage and 0.4% in FP32 (lbm3_strip.cuh).
 //
 // Multiplications and additions are fused where written, not by the compiler.
 #pragma once
@@ -108,12 +122,24 @@ __device__ __forceinline__ void stencils2(const float2 (&C)[4], const float2 (&N
   o.lap = make_float2(lap[0], lap[1]);
 }
 
-// One population pair (c, -c): f*_{+-} = om f + s +- v (see above).
+// x / 18 and x / 6 without the rounding of the constants.
+__device__ __forceinline__ float2 over18(float2 x) {
+  constexpr float c = 1.0f / 18.0f;
+  return fma2(x, both(c), mul2(x, both((float)(1.0 / 18.0 - (double)c))));
+}
+__device__ __forceinline__ float2 over6(float2 x) {
+  constexpr float c = 1.0f / 6.0f;
+  return fma2(x, both(c), mul2(x, both((float)(1.0 / 6.0 - (double)c))));
+}
+
+// One population pair (c, -c): f*_{+-} = f + (s - w_f S/2) +- (v - w_f D/2), S
+// and D the pair's sum and difference (see above; wh = -w_f/2).
 __device__ __forceinline__ void pair_f2(float2& fp, float2& fm, float2 cu, float2 cR, float2 v,
-                                        float2 k, float2 A, float2 om) {
-  const float2 s = fma2(cu, fma2(k, cu, cR), A);
-  fp = fma2(om, fp, add2(s, v));
-  fm = fma2(om, fm, sub2(s, v));
+                                        float2 k, float2 A, float2 wh) {
+  const float2 S = add2(fp, fm), D = sub2(fp, fm);
+  const float2 e = fma2(wh, S, fma2(cu, fma2(k, cu, cR), A)), o = fma2(wh, D, v);
+  fp = add2(fp, add2(e, o));
+  fm = add2(fm, sub2(e, o));
 }
 
 // Both collisions at two nodes (node3, kModeStep).  Returns a value that is
@@ -162,30 +188,33 @@ __device__ __forceinline__ float2 node3_pair(const Args3<float, S>& a, float2 (&
     wf = make_float2(N3<float>::rcp(tau.x), N3<float>::rcp(tau.y));
     hf = fma2(both(-0.5f), wf, one);
   }
-  const float2 om = sub2(one, wf);
-  wf = sub2(one, om);
   // rest population: f_eq,0 = (w0 - 1) p / c_s^2 + rho s_0 = -2p - rho u^2/2; F_0 = 0
-  F[0] = fma2(om, F[0], mul2(wf, fma2(both(-2.0f), p, mul2(both(-0.5f), ru2))));
+  F[0] = fma2(wf, sub2(fma2(both(-2.0f), p, mul2(both(-0.5f), ru2)), F[0]), F[0]);
+  const float2 wh = mul2(both(-0.5f), wf);
+  // the pairs' sums and differences are formed again below: kept, their 36
+  // registers spill at three CTAs per SM
+#pragma unroll
+  for (int i = 1; i < 19; ++i) asm volatile("" : "+f"(F[i].x), "+f"(F[i].y));
   const float2 base = fma2(both(3.0f), p, mul2(both(-1.5f), ru2));
-  const float2 wr = mul2(wf, rho), sixth = both(1.0f / 6.0f);
-  const float2 h6 = mul2(sixth, hf), w6 = mul2(sixth, wr);  // 3 w h_f, 3 w w_f rho, w = 1/18
-  float2 A = mul2(mul2(both(1.0f / 18.0f), wf), base);
-  float2 k = mul2(both(0.25f), wr);  // 4.5 w w_f rho
+  const float2 h6 = mul2(both(1.0f / 6.0f), hf);  // 3 w h_f, w = 1/18
+  float2 A = mul2(wf, over18(base));
+  float2 k = mul2(both(0.25f), mul2(wf, rho));  // 4.5 w w_f rho
   float2 rx = mul2(h6, Rx), ry = mul2(h6, Ry), rz = mul2(h6, Rz);
-  float2 vx = fma2(w6, ux, mul2(h6, Fx)), vy = fma2(w6, uy, mul2(h6, Fy)),
-         vz = fma2(w6, uz, mul2(h6, Fz));
-  pair_f2(F[1], F[2], ux, rx, vx, k, A, om);
-  pair_f2(F[3], F[4], uy, ry, vy, k, A, om);
-  pair_f2(F[5], F[6], uz, rz, vz, k, A, om);
+  float2 vx = over6(fma2(wf, mul2(rho, ux), mul2(hf, Fx))),
+         vy = over6(fma2(wf, mul2(rho, uy), mul2(hf, Fy))),
+         vz = over6(fma2(wf, mul2(rho, uz), mul2(hf, Fz)));
+  pair_f2(F[1], F[2], ux, rx, vx, k, A, wh);
+  pair_f2(F[3], F[4], uy, ry, vy, k, A, wh);
+  pair_f2(F[5], F[6], uz, rz, vz, k, A, wh);
   A = mul2(half, A), k = mul2(half, k);  // w = 1/36
   rx = mul2(half, rx), ry = mul2(half, ry), rz = mul2(half, rz);
   vx = mul2(half, vx), vy = mul2(half, vy), vz = mul2(half, vz);
-  pair_f2(F[7], F[8], add2(ux, uy), add2(rx, ry), add2(vx, vy), k, A, om);
-  pair_f2(F[9], F[10], sub2(ux, uy), sub2(rx, ry), sub2(vx, vy), k, A, om);
-  pair_f2(F[11], F[12], add2(ux, uz), add2(rx, rz), add2(vx, vz), k, A, om);
-  pair_f2(F[13], F[14], sub2(ux, uz), sub2(rx, rz), sub2(vx, vz), k, A, om);
-  pair_f2(F[15], F[16], add2(uy, uz), add2(ry, rz), add2(vy, vz), k, A, om);
-  pair_f2(F[17], F[18], sub2(uy, uz), sub2(ry, rz), sub2(vy, vz), k, A, om);
+  pair_f2(F[7], F[8], add2(ux, uy), add2(rx, ry), add2(vx, vy), k, A, wh);
+  pair_f2(F[9], F[10], sub2(ux, uy), sub2(rx, ry), sub2(vx, vy), k, A, wh);
+  pair_f2(F[11], F[12], add2(ux, uz), add2(rx, rz), add2(vx, vz), k, A, wh);
+  pair_f2(F[13], F[14], sub2(ux, uz), sub2(rx, rz), sub2(vx, vz), k, A, wh);
+  pair_f2(F[15], F[16], add2(uy, uz), add2(ry, rz), add2(vy, vz), k, A, wh);
+  pair_f2(F[17], F[18], sub2(uy, uz), sub2(ry, rz), sub2(vy, vz), k, A, wh);
 
   // ---- phase field: SRT limit of Eq. 33 on D3Q7 (c_s^2 = 1/4) ----
   J[0] = mul2(phi, ux), J[1] = mul2(phi, uy), J[2] = mul2(phi, uz);
@@ -202,8 +231,8 @@ __device__ __forceinline__ float2 node3_pair(const Args3<float, S>& a, float2 (&
   const float2 Vz = fma2(sh, N.qz, sub2(J[2], jp[2]));
   // movers: g + w_g (w_i (hbar + lambda phi) +- (1/2) c.J - g) +- h_g (1/2) c.V, the
   // small differences first: one rounding at the size of g (the phase field
-  // keeps what it rounds; with the complement as for f, phi's error after 200
-  // steps of a 256^3 column is 5.3e-8, so 5.0e-8)
+  // keeps what it rounds; with a complement 1 - w_g phi's error after 200 steps of
+  // a 256^3 column is 5.3e-8, so 5.0e-8)
   const float2 L8 = mul2(both(0.125f), fma2(both(a.lambda), phi, mu));
   float2 H[7];
   auto movers = [&](float2 gp, float2 gm, float2 Jc, float2 V, float2& hp, float2& hm) {

@@ -31,11 +31,13 @@
 // instruction).  A thread's 11 (FP16) or 18 (FP32) chunk copies are 128-thread
 // wide.  Per node 703 -> 557 instructions in FP16 storage, 642 -> 532 in FP32.
 // Measured, 256 x 256 x 512, MLUPS, bulk copies -> chunk copies: FP16 64 x 4 x
-// 32 with three CTAs per SM 31,300 -> 38,470 (0.73 of measured HBM), 64 x 2 x
-// 64 25,270 -> 34,450, with three stages and two CTAs 24,930 -> 34,530; FP32
-// 64 x 4 x 64 22,060 -> 24,290 (0.83).  One node per thread, not packed, with
-// bulk copies: FP16 28,300, FP32 22,200.  What bounds it now: HBM in FP32; in
-// FP16 issue (51%) and the latency of shared loads at 12 warps per SM.
+// 32 with three CTAs per SM 31,300 -> 38,470, 64 x 2 x 64 25,270 -> 34,450, with
+// three stages and two CTAs 24,930 -> 34,530; FP32 64 x 4 x 64 22,060 -> 24,290.
+// One node per thread, not packed, with bulk copies: FP16 28,300, FP32 22,200.
+// Now, with the collision in difference form (lbm3_pair.cuh; 573 and 544
+// instructions per node): FP16 37,900 (0.72 of measured HBM), 34,730 and 33,760,
+// FP32 24,270 (0.83).  What bounds it: HBM in FP32; in FP16 issue (51%) and the
+// latency of shared loads at 12 warps per SM.
 //
 // Every wait is bounded (wait_cycles); on expiry the CTA raises
 // kFlagTimeout3, waits (bounded by lbmk::kWaitCycles) for its own copies in
