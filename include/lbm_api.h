@@ -191,8 +191,9 @@ int32_t lbm_get_row_chains(const lbm_handle* h);
 /* Bound of the device waits, in SM clock cycles: the staged kernel's
  * waits for its staged rows, the chip-resident kernel's waits for its
  * neighbours' rims and the persistent kernel's grid barrier.  A
- * wait that gives up raises LBM_ERR_TIMEOUT (reported by the next
- * synchronising call or lbm_status); the kernel first waits, with the
+ * wait that gives up raises LBM_ERR_TIMEOUT (reported by lbm_fields,
+ * lbm_get_state, lbm_save, lbm_volume, lbm_adjoint_take_param_grads and, which
+ * clears it, lbm_status); the kernel first waits, with the
  * default bound, for the copies it issued, then returns, and the step's
  * results are not valid.  cycles < 0 restores the default, about 2 s
  * (4e9 cycles); 0 gives up at the first poll that finds the data missing
@@ -376,9 +377,11 @@ int lbm_record_steps(lbm_handle* h, int64_t count, void* d_states, int64_t strid
  *     [ny][nx] and d_u0 ([2][ny][nx] or NULL) are FP64 device copies of the
  *     initial fields, and d_adj_phi0 is FP64 whatever the precision.
  *   lbm_adjoint_take_param_grads: adds the accumulated parameter derivatives
- *     to h_param_grads[6] and clears the accumulator (synchronises).
+ *     to h_param_grads[6] and clears the accumulator (synchronises).  After a
+ *     wait that gave up: LBM_ERR_TIMEOUT, and h_param_grads and the accumulator
+ *     stay as they are, without that sweep's derivatives.
  * Synchronise when h_param_grads is non-NULL.  Errors: LBM_ERR_ARG (batch,
- * null buffers), LBM_ERR_WORKSPACE (no scratch), LBM_ERR_CUDA. */
+ * null buffers), LBM_ERR_WORKSPACE (no scratch), LBM_ERR_TIMEOUT, LBM_ERR_CUDA. */
 size_t lbm_adjoint_workspace_bytes(const lbm_handle* h);
 int lbm_adjoint_attach(lbm_handle* h, void* d_scratch, size_t bytes);
 int lbm_adjoint_seed_phi(lbm_handle* h, const double* d_dphi, void* d_adj_state);

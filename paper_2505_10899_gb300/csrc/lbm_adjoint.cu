@@ -37,6 +37,7 @@
 namespace lbmk {
 int set_last_error(int code, const char* msg);
 void drop_graphs(lbm_handle* h);
+int synced_valid(lbm_handle* h);
 }  // namespace lbmk
 
 using lbmk::CaseDev;
@@ -777,6 +778,14 @@ __global__ void ad_sum_partials(double* __restrict__ part, int nb, double* __res
   if (lane == 0) acc[q] += v;
 }
 
+// Parameter sums of a chip-resident sweep into the partials, unless a wait gave
+// up: its CTAs stop at different steps, and only whole sweeps count.
+__global__ void ad_commit(const double* __restrict__ pend, int n, double* __restrict__ part,
+                          const int32_t* __restrict__ flags) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n && !(*flags & lbmk::kFlagTimeout)) part[k] += pend[k];
+}
+
 // Scratch layout inside the caller's adjoint workspace: 19 planes of n
 // values in the handle's precision (phi, psi, 9 phi-stencil and 8
 // psi-stencil adjoints), then the FP64 per-block partials and accumulators.
@@ -785,8 +794,9 @@ struct AdScratch {
   void *phi, *psi, *lP, *lQ;
   double *part, *sums;
   double *init_lphi, *init_llap;
-  lbmk::ResTile* tiles;  // chip-resident sweep: tiles, two sets of exchange slots
-  uint4* slots;
+  lbmk::ResTile* tiles;  // chip-resident sweep: tiles, two sets of exchange slots,
+  uint4* slots;          // parameter sums of the sweep in flight (by CTA)
+  double* pend;
 };
 
 size_t elem_bytes(const lbm_handle* h) { return h->precision == LBM_F64 ? 8 : 4; }
@@ -804,7 +814,8 @@ size_t tile_bytes(const lbmk::ResPlan& p) {
 
 size_t scratch_bytes(const lbm_handle* h, const lbmk::ResPlan& p) {
   const int64_t n = (int64_t)h->params[0].nx * h->params[0].ny;
-  return base_bytes(n, elem_bytes(h)) + tile_bytes(p) + (size_t)2 * p.nslots * sizeof(uint4);
+  return base_bytes(n, elem_bytes(h)) + tile_bytes(p) + (size_t)2 * p.nslots * sizeof(uint4) +
+         p.tiles.size() * kNParam * sizeof(double);
 }
 
 AdScratch carve(lbm_handle* h) {
@@ -823,6 +834,7 @@ AdScratch carve(lbm_handle* h) {
   char* r = b + base_bytes(n, es);
   s.tiles = (lbmk::ResTile*)r;
   s.slots = (uint4*)(r + tile_bytes(h->adj_res));
+  s.pend = (double*)(s.slots + (size_t)2 * h->adj_res.nslots);
   return s;
 }
 
@@ -853,8 +865,11 @@ int take_grads(lbm_handle* h, double* out) {
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(raw, s.sums, sizeof raw, cudaMemcpyDeviceToHost, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(s.sums, 0, sizeof raw, h->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
+  // after a wait that gave up nothing is handed out, and what the sweeps
+  // before it accumulated stays
+  if (int rc = lbmk::synced_valid(h)) return rc;
+  e = cudaMemsetAsync(s.sums, 0, sizeof raw, h->stream);
   if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
   to_param_grads(h->params[0], raw, out);
   return LBM_OK;
@@ -1007,6 +1022,8 @@ int run_sweep(lbm_handle* h, const float* states, int64_t stride, int32_t count,
   AdScratch s = carve(h);
   const AdArgs<float> a = ad_args<float>(h, s, 0);
   const lbmk::ResTile* tiles = s.tiles;
+  const int nsums = (int)h->adj_res.tiles.size() * kNParam;
+  int first = 1;
   while (count > 0) {
     const int32_t cnt = count < kChunk ? count : kChunk;
     if (h->adj_epoch > UINT32_MAX - 2 * kChunk) {  // tags run out: start over
@@ -1024,6 +1041,9 @@ int run_sweep(lbm_handle* h, const float* states, int64_t stride, int32_t count,
     r.nslots = h->adj_res.nslots;
     r.slots = s.slots;
     r.adj = adj;
+    r.pend = s.pend;
+    r.first = first;
+    first = 0;
     r.wait_cycles = h->wait_cycles;
     r.flags = h->flags;
     h->adj_epoch += (uint32_t)cnt;
@@ -1034,6 +1054,9 @@ int run_sweep(lbm_handle* h, const float* states, int64_t stride, int32_t count,
     if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
     count -= cnt;
   }
+  ad_commit<<<(nsums + 255) / 256, 256, 0, h->stream>>>(s.pend, nsums, s.part, h->flags);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
   return LBM_OK;
 }
 

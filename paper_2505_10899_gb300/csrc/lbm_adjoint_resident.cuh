@@ -23,7 +23,8 @@
 //
 // Parameter terms: per step and warp as in ad_node (R within a warp); the
 // warp sums accumulate in FP64, lane q of a warp holding parameter q, and
-// enter the CTA's slots in warp order at the end.
+// enter the CTA's slots in warp order at the end.  They count only if no wait of
+// the sweep gave up (ad_commit).
 //
 // Measured, us per adjoint step (two launches per step -> here): 512 x 256 with
 // walls 23.9 -> 11.6, 384 x 192 21.8 -> 7.8, 201 x 101 with walls 22.6 -> 4.9,
@@ -57,6 +58,8 @@ struct AdRun {
   uint4* slots;
   int prefetch;          // the launch's states exceed what L2 keeps
   float* adj;            // adjoint of S_{t0 + count} in, of S_{t0} out
+  double* pend;          // [CTAs][kNParam] parameter sums, added to by launches
+  int first;             // of one sweep after the first
   long long wait_cycles;
   int32_t* flags;
 };
@@ -435,6 +438,7 @@ __global__ void __launch_bounds__(kAdNT, 1)
   if (tid < kNParam) {
     double v = 0.0;
     for (int q = 0; q < kAdNT / 32; ++q) v += red[q][tid];
-    a.part[(int64_t)blockIdx.x * kNParam + tid] += v;
+    double* const s = run.pend + (int64_t)blockIdx.x * kNParam + tid;
+    *s = run.first ? v : *s + v;
   }
 }

@@ -684,12 +684,16 @@ int flags_status(int32_t fl) {
   return LBM_OK;
 }
 
-int read_flags(lbm_handle* h) {
+int read_flags(lbm_handle* h, int32_t mask = -1) {
   int32_t fl = 0;
   LBM_CUDA(cudaMemcpyAsync(&fl, h->flags, sizeof fl, cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(cudaStreamSynchronize(h->stream));
-  return flags_status(fl);
+  return flags_status(fl & mask);
 }
+
+// Synchronises; an error if a device wait gave up, so that what the call
+// copied out is not valid.
+int sync_valid(lbm_handle* h) { return read_flags(h, lbmk::kFlagTimeout); }
 
 // Volumes of every case into `out` (device).  flags_out: where the one-launch
 // form leaves a copy of the error flags; *fused says whether it ran.  One
@@ -753,8 +757,7 @@ int do_fields(lbm_handle* h, int c, double* phi, double* ux, double* uy, double*
     if (outs[q])
       LBM_CUDA(cudaMemcpyAsync(outs[q], st + q * n, n * sizeof(double), cudaMemcpyDefault,
                                h->stream));
-  LBM_CUDA(cudaStreamSynchronize(h->stream));
-  return LBM_OK;
+  return sync_valid(h);
 }
 
 template <typename T>
@@ -787,7 +790,7 @@ int do_get_state(lbm_handle* h, int c, double* f, double* g, double* j) {
       LBM_CUDA(cudaStreamSynchronize(h->stream));
     }
   }
-  return LBM_OK;
+  return sync_valid(h);
 }
 
 template <typename T>
@@ -891,6 +894,7 @@ int retile(lbm_handle* h, const Tiling& t, int nchains) {
 namespace lbmk {
 int set_last_error(int code, const char* msg) { return fail(code, msg); }
 void drop_graphs(lbm_handle* h) { drop_graph(h); }
+int synced_valid(lbm_handle* h) { return sync_valid(h); }
 }  // namespace lbmk
 
 // ============================================================================
@@ -1504,8 +1508,7 @@ int lbm_save(lbm_handle* h, void* h_buf, size_t bytes) {
       p += n * es;
     }
   }
-  LBM_CUDA(cudaStreamSynchronize(h->stream));
-  return LBM_OK;
+  return sync_valid(h);
 }
 
 int lbm_load(lbm_handle* h, const void* h_buf, size_t bytes) {
