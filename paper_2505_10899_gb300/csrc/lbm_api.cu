@@ -1232,7 +1232,9 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
   }
   // Trial launches read the current source buffers and write the other
   // buffer set (populations and phi*u), which the next real step overwrites
-  // completely: the state is not changed and the clock does not advance.
+  // completely: the state is not changed and the clock does not advance.  (A
+  // trial of the chip-resident kernel runs on from the state on the chip, and
+  // writes and flags nothing.)
   // lbm_step replays the step kernels of variants 1 and 2 as CUDA graphs
   // (one branch per chain): time their trials the same way, as one captured
   // graph of n steps (replayed once untimed, then timed).  At least 8 trial

@@ -99,7 +99,7 @@ constexpr int kResMaxSteps = 1024;  // steps of one launch
 // One launch of the chip-resident kernel.
 struct ResRun {
   int32_t nsteps;      // 1 .. kResMaxSteps
-  int32_t store;       // 0: leave the state as it is (autotuning trials)
+  int32_t store;       // 0: leave the state and its non-finite flag as they are (autotuning trials)
   uint32_t epoch;      // tag of the first exchange, unique over the handle's launches
   uint32_t nslots;     // exchange slots of one set (two sets)
   void* slots;

@@ -432,7 +432,8 @@ __global__ void __launch_bounds__(NT, MINB)
 #pragma unroll
         for (int i = 0; i < 9; ++i) nxt[(9 + i) * PC + c] = F[i];
       }
-      if (!isfinite(S.p + o.ux + o.uy + o.p)) atomicOr(a.flags, kFlagNonFinite);
+      // (a trial's later steps are not states of the handle)
+      if (!isfinite(S.p + o.ux + o.uy + o.p) && run.store) atomicOr(a.flags, kFlagNonFinite);
       if (run.rec && s + 1 < run.nsteps) record(s + 1, r, F, G);
     }
     if (s + 1 == run.nsteps) break;
