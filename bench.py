@@ -653,6 +653,7 @@ def run_extras(args, cases, dev):
             out["f64_first64cases"] = {
                 "mlups": out["f64_mlups_first64cases"], "ms_per_step": round(ms / 20, 4),
                 "tiling": list(s.tiling()[:2]), "kernel": s.kernel(),
+                "chip_resident": s.resident(),
                 "roofline": fp64_roofline("coupled_step_f64_batched16", nodes, ms / 20,
                                           out["fp64_peak"])}
         s.close()
@@ -677,7 +678,9 @@ def run_extras(args, cases, dev):
         ms = timed(s, 16384)
         phi = s.fields(0)[0]
         fin[prec] = phi
-        vort[f"{prec}_kernel"] = {"variant": s.kernel(), "bx": s.tiling()[0], "rows": s.tiling()[1]}
+        vort[f"{prec}_kernel"] = ("step_resident" if s.resident() else
+                                  {"variant": s.kernel(), "bx": s.tiling()[0],
+                                   "rows": s.tiling()[1]})
         vort[f"{prec}_mlups"] = round(256 * 256 * 16384 / (ms * 1e-3) / 1e6, 1)
         vort[f"{prec}_shape_error"] = float(np.abs(phi - vphi0).sum() / vphi0.sum())
         vort[f"{prec}_volume_drift"] = float(s.volume()[0] / v0 - 1.0)
@@ -989,7 +992,8 @@ def adjoint_sweep_timing(dev, precisions=("f32", "f64"), nrec=256):
         out[prec] = {"forward_us_per_step": round(fwd * 1e3, 2),
                      "adjoint_us_per_step": round(adj_ms * 1e3, 2),
                      "adjoint_over_forward": round(adj_ms / fwd, 3),
-                     "forward_kernel": a.sim.kernel(), "forward_tiling": list(a.sim.tiling()),
+                     "forward_kernel": "step_resident" if a.sim.resident() else a.sim.kernel(),
+                     "forward_tiling": None if a.sim.resident() else list(a.sim.tiling()),
                      "status": a.sim.status()}
         a.close()
         del rec, adj, spare
@@ -1025,9 +1029,11 @@ def shear_timing(dev, nsteps=20000, ckpt=256, grad_steps=20000):
         ms = a.elapsed_time(b) / (nsteps - 3)
         phi = torch.as_tensor(s.fields(0)[0])
         out[prec] = {"mlups": round(512 * 256 / (ms * 1e-3) / 1e6, 1),
-                     "tiling": {"bx": s.tiling()[0], "rows": s.tiling()[1]},
-                     "kernel": {1: "step_kernel", 3: "step_kernel_persistent"}.get(s.kernel(),
-                                                                                    "?"),
+                     "tiling": (None if s.resident() else
+                                {"bx": s.tiling()[0], "rows": s.tiling()[1]}),
+                     "kernel": ("step_resident" if s.resident() else
+                                {1: "step_kernel", 2: "step_kernel_tma",
+                                 3: "step_kernel_persistent"}[s.kernel()]),
                      "taylor_D": float(A.taylor_deformation(phi)),
                      "status": s.status()}
         s.close()

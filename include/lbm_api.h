@@ -255,10 +255,16 @@ int lbm_set_tiling(lbm_handle* h, int32_t bx, int32_t rows);
 /* Self-tuning: time every (kernel variant, bx, rows) candidate on this
  * batch with max(trials, 8) trial steps each (CUDA events on the handle's
  * stream) and keep the fastest.  The step kernels of variants 1 and 2 are
- * timed as a captured CUDA graph of those steps, as lbm_step replays them;
- * variant 3 as one persistent launch.  Trial launches read the current
- * state and write only the buffers the next step overwrites, so the state
- * and the step index do not change.  Outputs may be NULL.  Synchronises. */
+ * timed as a captured CUDA graph of those steps, as lbm_step replays them.
+ * Where the batch fits the chip-resident kernel (see lbm_step) that is timed
+ * too, and kept or left for longer runs (from 1 to 4 steps on, as measured)
+ * beside the fastest of variants 1 and 2, which serves the others (shorter runs,
+ * tracked volumes, captured streams) and is what best_kernel, best_bx, best_rows and lbm_get_kernel report; best_ms is
+ * the fastest of all, and lbm_get_resident says which it was.  Elsewhere variant
+ * 3 is timed as one persistent launch, unless volumes are tracked.  Trial
+ * launches read the current state and write only the buffers the next step
+ * overwrites, so the state, the step index and the error flags do not change.
+ * Outputs may be NULL.  Synchronises. */
 int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel,
                  int32_t* best_bx, int32_t* best_rows, double* best_ms);
 
@@ -269,11 +275,13 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel,
  * kernel where the batch fits it, see lbm_step, else a grid barrier between
  * steps).  All run the same per-node arithmetic (equal up to rounding, see
  * lbm_set_tiling).  lbm_get_kernel returns the variant of single steps in use
- * (1 or 2, or 3 if asked for).
+ * (1 or 2, or 3 if asked for); lbm_get_resident the steps from which on a run
+ * takes the chip-resident kernel as the handle stands (4 before tuning), or 0.
  * Changing the variant rebuilds the work-item table (whole-row chains run
  * the staged kernel only; synchronises). */
 int lbm_set_kernel(lbm_handle* h, int32_t variant);
 int32_t lbm_get_kernel(const lbm_handle* h);
+int32_t lbm_get_resident(const lbm_handle* h);
 
 /* Total number of volume regions over all cases. */
 int32_t lbm_num_regions(const lbm_handle* h);

@@ -481,14 +481,17 @@ bool res_allowed(const lbm_handle* h) {
   return h->res.variant >= 0 && (!h->pd.plain || h->tma_ok);
 }
 
-// Whether a run of nsteps steps takes the chip-resident kernel: the batch
-// fits, no other kernel was asked for, no per-step volumes are tracked, and
-// the stream is not being captured (a replayed launch would reuse its tags).
-constexpr int64_t kResMinSteps = 4;
+// Whether long runs take it now: no other kernel was asked for or measured
+// faster, and no per-step volumes are tracked.
+bool res_chosen(const lbm_handle* h) {
+  return res_allowed(h) && !h->track && (h->res_auto || h->kernel == 3);
+}
+
+// Whether a run of nsteps steps takes it: enough steps to pay for loading and
+// storing the state, and a stream that is not being captured (a replayed launch
+// would reuse its tags).
 bool use_resident(const lbm_handle* h, int64_t nsteps) {
-  if (!res_allowed(h) || h->track || (h->kernel != 0 && h->kernel != 3) ||
-      nsteps < (h->kernel == 3 ? 1 : kResMinSteps))
-    return false;
+  if (!res_chosen(h) || nsteps < (h->kernel == 3 ? 1 : h->res_min)) return false;
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
     cudaGetLastError();  // another stream's capture forbids the query
@@ -498,17 +501,17 @@ bool use_resident(const lbm_handle* h, int64_t nsteps) {
 }
 
 // nsteps (at most kResMaxSteps) steps in one launch of the chip-resident
-// kernel.  store = false: the state is left as it is (autotuning trials).
+// kernel.  store: see ResRun (0 and 2 in autotuning trials).
 // rec: the states entering each step are recorded, `stride` bytes apart.
 template <typename T>
-int launch_res(lbm_handle* h, int nsteps, bool store, void* rec, int64_t stride) {
+int launch_res(lbm_handle* h, int nsteps, int store, void* rec, int64_t stride) {
   if (h->res_epoch > UINT32_MAX - 2 * lbmk::kResMaxSteps) {  // tags run out: start over
     LBM_CUDA(cudaMemsetAsync(h->ws + h->L.rslots, 0, h->L.rslot_bytes, h->stream));
     h->res_epoch = 1;
   }
   lbmk::ResRun r{};
   r.nsteps = nsteps;
-  r.store = store ? 1 : 0;
+  r.store = store;
   r.epoch = h->res_epoch;
   r.nslots = h->res.nslots;
   r.slots = h->ws + h->L.rslots;
@@ -528,8 +531,8 @@ int launch_res(lbm_handle* h, int nsteps, bool store, void* rec, int64_t stride)
 int run_resident(lbm_handle* h, int64_t nsteps, void* rec = nullptr, int64_t stride = 0) {
   while (nsteps > 0) {
     const int cnt = (int)std::min<int64_t>(nsteps, lbmk::kResMaxSteps);
-    const int rc = h->precision == LBM_F32 ? launch_res<float>(h, cnt, true, rec, stride)
-                                           : launch_res<double>(h, cnt, true, rec, stride);
+    const int rc = h->precision == LBM_F32 ? launch_res<float>(h, cnt, 1, rec, stride)
+                                           : launch_res<double>(h, cnt, 1, rec, stride);
     if (rc) return rc;
     if (rec) rec = (char*)rec + cnt * stride;
     h->parity ^= (cnt & 1);
@@ -1204,18 +1207,29 @@ int lbm_set_kernel(lbm_handle* h, int32_t variant) {
     return fail(LBM_ERR_ARG, "bulk-copy kernel needs nx a multiple of 16 bytes and nx >= 4");
   if (variant == 3 && total_nodes(h) > kPersistMaxNodes)
     return fail(LBM_ERR_ARG, "persistent kernel is for batches of at most 4 Mi nodes");
-  if (variant == h->kernel) return LBM_OK;
-  const int keep = h->kernel;
-  h->kernel = variant;
-  const int rc = retile(h, h->tile, h->chains_req);  // whole-row chains follow the kernel
-  if (rc != LBM_OK) h->kernel = keep;
-  return rc;
+  if (variant != h->kernel) {
+    const int keep = h->kernel;
+    h->kernel = variant;
+    const int rc = retile(h, h->tile, h->chains_req);  // whole-row chains follow the kernel
+    if (rc != LBM_OK) {
+      h->kernel = keep;
+      return rc;
+    }
+  }
+  h->res_auto = variant == 0 || variant == 3;
+  h->res_min = lbmk::kResMinSteps;
+  return LBM_OK;
 }
 
 int32_t lbm_get_kernel(const lbm_handle* h) {
   if (!h) return -1;
   if (h->kernel == 3) return 3;
   return use_tma(h) ? 2 : 1;
+}
+
+int32_t lbm_get_resident(const lbm_handle* h) {
+  if (!h || !res_chosen(h)) return 0;
+  return h->kernel == 3 ? 1 : h->res_min;
 }
 
 int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* best_bx,
@@ -1251,7 +1265,9 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
   int rc = LBM_OK;
   for (int kv : {2, 1, 3}) {
     if (kv == 2 && !h->tma_ok) continue;
-    if (kv == 3 && total_nodes(h) > kPersistMaxNodes) continue;
+    // (the grid-barrier kernel: where the chip-resident one, tried below, cannot
+    // run; steps with tracked volumes take neither)
+    if (kv == 3 && (total_nodes(h) > kPersistMaxNodes || res_allowed(h) || h->track)) continue;
     for (int bx : {128, 64, 32}) {
       for (int rows : {2, 4, 8, 16, 32, 64, 128}) {
         // whole-row chains exist for the FP32 staged kernel on 128-wide
@@ -1262,21 +1278,8 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
           h->row_chains = rcv == 1;
           rc = lbm_set_tiling(h, bx, rows);
           if (rc != LBM_OK) break;
-          int n_run = n_trial;
           cudaError_t e = cudaSuccess;
-          if (kv == 3 && res_allowed(h)) {
-            // the chip-resident kernel has tiles of its own: one trial
-            if (bx != 128 || rows != 2) continue;
-            n_run = std::max(n_trial, kGraphSteps);
-            auto trial = [&]() {
-              return h->precision == LBM_F32 ? launch_res<float>(h, n_run, false, nullptr, 0)
-                                             : launch_res<double>(h, n_run, false, nullptr, 0);
-            };
-            rc = trial();
-            if (rc == LBM_OK) e = cudaEventRecord(e0, h->stream);
-            if (rc == LBM_OK && e == cudaSuccess) rc = trial();
-            if (rc != LBM_OK) break;
-          } else if (kv == 3) {  // one launch of n_trial steps without flipping buffers
+          if (kv == 3) {  // one launch of n_trial steps without flipping buffers
             rc = launch_persist(h, h->stream, h->parity, 1, 0);
             if (rc == LBM_OK) e = cudaEventRecord(e0, h->stream);
             if (rc == LBM_OK && e == cudaSuccess) rc = launch_persist(h, h->stream, h->parity, n_trial, 0);
@@ -1300,11 +1303,10 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
             rc = fail(LBM_ERR_CUDA, std::string("autotune: ") + cudaGetErrorString(e));
             break;
           }
-          if (ms / n_run < best) {
-            best = ms / n_run;
+          if (ms / n_trial < best) {
+            best = ms / n_trial;
             best_t.bx = bx;
             best_t.rows = rows;
-            if (kv == 3 && res_allowed(h)) best_t = keep_tile;
             best_k = kv;
             best_rc = rcv == 1;
           }
@@ -1315,6 +1317,54 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
     }
     if (rc != LBM_OK) break;
   }
+  // The chip-resident kernel has tiles of its own.  Whether it is faster, and
+  // from how many steps on, is kept beside the best of variants 1 and 2, which
+  // go on to serve what it does not: shorter runs, tracked volumes, captured
+  // streams.
+  bool res = h->res_auto;
+  int res_min = h->res_min;
+  if (rc == LBM_OK && res_allowed(h) && !h->track) {
+    h->kernel = best_k;
+    h->row_chains = best_rc;
+    rc = lbm_set_tiling(h, best_t.bx, best_t.rows);
+    // ms of one of `reps` equal launches, after an untimed one
+    auto timed = [&](int reps, float* ms, auto&& launch) -> int {
+      int r = launch();
+      cudaError_t e = r == LBM_OK ? cudaEventRecord(e0, h->stream) : cudaSuccess;
+      for (int k = 0; k < reps && r == LBM_OK; ++k) r = launch();
+      if (r != LBM_OK) return r;
+      if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
+      if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+      if (e == cudaSuccess) e = cudaEventElapsedTime(ms, e0, e1);
+      *ms /= (float)reps;
+      return e == cudaSuccess ? LBM_OK
+                              : fail(LBM_ERR_CUDA, std::string("autotune: ") + cudaGetErrorString(e));
+    };
+    auto resident = [&](int n, int store) {
+      return h->precision == LBM_F32 ? launch_res<float>(h, n, store, nullptr, 0)
+                                     : launch_res<double>(h, n, store, nullptr, 0);
+    };
+    const int n_run = std::max(n_trial, kGraphSteps);
+    float ms = 0.f;
+    if (rc == LBM_OK) rc = timed(1, &ms, [&] { return resident(n_run, 0); });
+    if (rc == LBM_OK) {
+      res = ms / n_run < best;
+      if (res) best = ms / n_run;
+    }
+    if (rc == LBM_OK && res) {  // calls of 1 and 3 steps; 2 lies between
+      float r[2], d[2];
+      for (int q = 0; q < 2 && rc == LBM_OK; ++q) {
+        const int n = 1 + 2 * q;
+        rc = timed(16, &r[q], [&] { return resident(n, 2); });
+        if (rc == LBM_OK)
+          rc = timed(16, &d[q],
+                     [&] { return enqueue_steps(h, h->stream, h->parity, n, false, false, true); });
+      }
+      if (rc == LBM_OK) rc = set_clock(h);
+      res_min = lbmk::kResMinSteps;
+      if (rc == LBM_OK && r[1] < d[1]) res_min = r[0] < d[0] ? 1 : (r[0] + r[1] < d[0] + d[1] ? 2 : 3);
+    }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (rc != LBM_OK) {
@@ -1324,6 +1374,8 @@ int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel, int32_t* b
     return rc;
   }
   h->kernel = best_k;
+  h->res_auto = res;
+  h->res_min = res_min;
   h->row_chains = best_rc;
   rc = lbm_set_tiling(h, best_t.bx, best_t.rows);
   if (rc != LBM_OK) return rc;

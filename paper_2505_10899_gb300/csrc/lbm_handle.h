@@ -90,9 +90,12 @@ struct lbm_handle {
   double* vol = nullptr;
   double* staging = nullptr;
   int64_t max_plane = 0;
-  // chip-resident kernel: tiles (none if the batch does not fit), and the tag
-  // of its next exchange
+  // chip-resident kernel: tiles (none if the batch does not fit), whether runs
+  // that it can serve take it and from how many steps on (autotuning measures
+  // both), and the tag of its next exchange
   lbmk::ResPlan res;
+  bool res_auto = true;
+  int res_min = lbmk::kResMinSteps;
   uint32_t res_epoch = 1;
   // reverse mode (lbm_adjoint_attach): caller-provided FP64 scratch
   char* adj_ws = nullptr;

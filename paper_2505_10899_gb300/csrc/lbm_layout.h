@@ -99,7 +99,10 @@ constexpr int kResMaxSteps = 1024;  // steps of one launch
 // One launch of the chip-resident kernel.
 struct ResRun {
   int32_t nsteps;      // 1 .. kResMaxSteps
-  int32_t store;       // 0: leave the state and its non-finite flag as they are (autotuning trials)
+  // 1: a run of the handle.  Autotuning trials leave the clock and the
+  // non-finite flag alone; 0 writes nothing, 2 the planes (an odd nsteps: those
+  // that the next step overwrites)
+  int32_t store;
   uint32_t epoch;      // tag of the first exchange, unique over the handle's launches
   uint32_t nslots;     // exchange slots of one set (two sets)
   void* slots;

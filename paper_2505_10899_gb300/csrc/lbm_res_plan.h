@@ -12,6 +12,8 @@
 namespace lbmk {
 
 constexpr int kResSMs = 152;
+// Steps that pay for loading and storing the state, where nothing was measured.
+constexpr int kResMinSteps = 4;
 constexpr int kResMinTile = 64;  // nodes: tiles of 32, 64 and 128 measure alike
 
 struct ResPlan {

@@ -433,7 +433,7 @@ __global__ void __launch_bounds__(NT, MINB)
         for (int i = 0; i < 9; ++i) nxt[(9 + i) * PC + c] = F[i];
       }
       // (a trial's later steps are not states of the handle)
-      if (!isfinite(S.p + o.ux + o.uy + o.p) && run.store) atomicOr(a.flags, kFlagNonFinite);
+      if (!isfinite(S.p + o.ux + o.uy + o.p) && run.store == 1) atomicOr(a.flags, kFlagNonFinite);
       if (run.rec && s + 1 < run.nsteps) record(s + 1, r, F, G);
     }
     if (s + 1 == run.nsteps) break;
@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(NT, MINB)
     }
     if (__syncthreads_or(bad)) {
       if (tid == 0) atomicOr(a.flags, kFlagTimeout);
-      if (run.store && blockIdx.x == 0 && tid == 0) *run.t_dev = run.t0 + run.nsteps;
+      if (run.store == 1 && blockIdx.x == 0 && tid == 0) *run.t_dev = run.t0 + run.nsteps;
       return;
     }
     phase_edge(nxt);
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(NT, MINB)
     store_node<T, COUPLED>(fd, gd, cdp->J[dst], cdp->g0lo[dst], P, gnode[r], F, G, lo[r], o,
                            a.flags, nn);
   }
-  if (blockIdx.x == 0 && tid == 0) *run.t_dev = run.t0 + run.nsteps;
+  if (run.store == 1 && blockIdx.x == 0 && tid == 0) *run.t_dev = run.t0 + run.nsteps;
 }
 
 }  // namespace lbmk

@@ -92,6 +92,7 @@ def _load():
                           ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32), _D],
                          ctypes.c_int),
         "lbm_get_kernel": ([_H], ctypes.c_int32),
+        "lbm_get_resident": ([_H], ctypes.c_int32),
         "lbm_fields": ([_H, ctypes.c_int32, _D, _D, _D, _D], ctypes.c_int),
         "lbm_get_state": ([_H, ctypes.c_int32, _D, _D, _D, ctypes.POINTER(ctypes.c_int64)],
                           ctypes.c_int),
@@ -508,6 +509,10 @@ class Sim:
 
     def kernel(self):
         return lbm_get_kernel(self.h)
+
+    def resident(self):
+        """Steps from which on a run takes the chip-resident kernel; 0: none does."""
+        return int(_lib.lbm_get_resident(self.h))
 
     def track_volume(self, enable=True):
         """Fused per-step volumes into a device tensor (one FP64 per case)."""
