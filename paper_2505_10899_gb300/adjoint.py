@@ -16,6 +16,8 @@ the device buffers.
 """
 from __future__ import annotations
 
+import contextlib
+
 import numpy as np
 import torch
 
@@ -60,14 +62,31 @@ class AdjointSim:
     def new_state(self):
         return torch.zeros((20,) + self.shape, dtype=self.dtype, device=self.dev)
 
+    @contextlib.contextmanager
+    def on_stream(self):
+        """Around library calls that read or write tensors: the handle's stream first waits
+        for the caller's (which may still fill them, or work on what their memory held
+        before), and the caller's then for the handle's (before it reads or frees them)."""
+        cur = torch.cuda.current_stream(self.dev)
+        other = cur != self.sim.stream
+        if other:
+            self.sim.stream.wait_stream(cur)
+        try:
+            yield
+        finally:
+            if other:
+                cur.wait_stream(self.sim.stream)
+
     def snapshot(self, buf=None):
         if buf is None:
             buf = torch.empty((self.planes,) + self.shape, dtype=self.dtype, device=self.dev)
-        lbm.lbm_snapshot(self.h, 0, buf.data_ptr())
+        with self.on_stream():
+            lbm.lbm_snapshot(self.h, 0, buf.data_ptr())
         return buf
 
     def restore(self, buf, t):
-        lbm.lbm_restore(self.h, 0, buf.data_ptr())
+        with self.on_stream():
+            lbm.lbm_restore(self.h, 0, buf.data_ptr())
         lbm.lbm_set_time(self.h, int(t))
 
     def step(self, n=1):
@@ -77,24 +96,17 @@ class AdjointSim:
     def t(self):
         return lbm.lbm_time(self.h)
 
-    def _after_current(self):
-        """Orders the handle's stream after the caller's: a new buffer may be memory
-        that the caller's stream still works on."""
-        cur = torch.cuda.current_stream(self.dev)
-        if cur != self.sim.stream:
-            self.sim.stream.wait_stream(cur)
-
     def phi(self):
         out = torch.empty(self.shape, dtype=torch.float64, device=self.dev)
-        self._after_current()
-        lbm.lbm_field_phi(self.h, 0, out.data_ptr())
+        with self.on_stream():
+            lbm.lbm_field_phi(self.h, 0, out.data_ptr())
         return out
 
     def seed_phi(self, dphi):
         adj = torch.empty((20,) + self.shape, dtype=self.dtype, device=self.dev)
         dphi = dphi.to(device=self.dev, dtype=torch.float64).contiguous()
-        self._after_current()
-        lbm.lbm_adjoint_seed_phi(self.h, dphi.data_ptr(), adj.data_ptr())
+        with self.on_stream():
+            lbm.lbm_adjoint_seed_phi(self.h, dphi.data_ptr(), adj.data_ptr())
         return adj
 
     def vjp_step(self, adj_in, grads=None, adj_out=None):
@@ -102,7 +114,8 @@ class AdjointSim:
         accumulate on the device; with ``grads`` (numpy[6]) they are fetched."""
         if adj_out is None:
             adj_out = torch.empty((20,) + self.shape, dtype=self.dtype, device=self.dev)
-        rc = lbm.lbm_adjoint_step(self.h, adj_in.data_ptr(), adj_out.data_ptr(), grads)
+        with self.on_stream():
+            rc = lbm.lbm_adjoint_step(self.h, adj_in.data_ptr(), adj_out.data_ptr(), grads)
         if rc != lbm.LBM_OK:
             raise lbm.LbmError(rc, "lbm_adjoint_step", lbm.lib().lbm_last_error().decode())
         return adj_out
@@ -113,8 +126,9 @@ class AdjointSim:
         derivatives accumulate on the device."""
         if adj_out is None:
             adj_out = torch.empty((20,) + self.shape, dtype=self.dtype, device=self.dev)
-        rc = lbm.lbm_adjoint_step_from(self.h, state.data_ptr(), int(t), adj_in.data_ptr(),
-                                       adj_out.data_ptr(), None)
+        with self.on_stream():
+            rc = lbm.lbm_adjoint_step_from(self.h, state.data_ptr(), int(t), adj_in.data_ptr(),
+                                           adj_out.data_ptr(), None)
         if rc != lbm.LBM_OK:
             raise lbm.LbmError(rc, "lbm_adjoint_step_from", lbm.lib().lbm_last_error().decode())
         return adj_out
@@ -123,11 +137,26 @@ class AdjointSim:
         lbm.lbm_adjoint_take_param_grads(self.h, grads)
 
     def vjp_init(self, adj_state, grads):
-        out = torch.zeros(self.shape, dtype=torch.float64, device=self.dev)
-        lbm.lbm_adjoint_init(self.h, self.phi0.data_ptr(),
-                             0 if self.u0 is None else self.u0.data_ptr(),
-                             adj_state.data_ptr(), out.data_ptr(), grads)
+        out = torch.empty(self.shape, dtype=torch.float64, device=self.dev)
+        with self.on_stream():
+            lbm.lbm_adjoint_init(self.h, self.phi0.data_ptr(),
+                                 0 if self.u0 is None else self.u0.data_ptr(),
+                                 adj_state.data_ptr(), out.data_ptr(), grads)
         return out
+
+    def record(self, states):
+        """Steps once per entry of ``states``, which receives the states entering the steps."""
+        with self.on_stream():
+            lbm.lbm_record_steps(self.h, len(states), states.data_ptr(),
+                                 states[0].numel() * states.element_size())
+
+    def sweep(self, states, t0, adj, spare):
+        """Adjoint of S_t0, in place of that of S_{t0 + len(states)} in ``adj``, over recorded
+        states; ``spare`` is scratch of its size."""
+        with self.on_stream():
+            lbm.lbm_adjoint_sweep(self.h, states.data_ptr(),
+                                  states[0].numel() * states.element_size(), t0, len(states),
+                                  adj.data_ptr(), spare.data_ptr())
 
     def close(self):
         self.sim.close()
@@ -170,7 +199,7 @@ class CoupledRun(torch.autograd.Function):
             if t < t_rec:
                 ckpts[t] = asim.snapshot()
         if m:  # snapshot and step, m times, in one library call
-            lbm.lbm_record_steps(asim.h, m, rec.data_ptr(), rec[0].numel() * rec.element_size())
+            asim.record(rec)
         phiT = asim.phi()
         ctx.asim, ctx.ckpts, ctx.rec, ctx.t_rec = asim, ckpts, rec, t_rec
         ctx.nsteps, ctx.k = nsteps, ckpt_every
@@ -187,21 +216,18 @@ class CoupledRun(torch.autograd.Function):
         spare = torch.empty_like(adj)
         # recorded states: no recomputation (one library call for the sweep)
         if nsteps > t_rec:
-            lbm.lbm_adjoint_sweep(asim.h, rec.data_ptr(), rec[0].numel() * rec.element_size(),
-                                  t_rec, nsteps - t_rec, adj.data_ptr(), spare.data_ptr())
+            asim.sweep(rec, t_rec, adj, spare)
         ctx.rec = rec = None
         # checkpointed segments below: recompute the states into one buffer,
         # then run the segment backwards
         if t_rec > 0:
             seg = torch.empty((min(k, t_rec),) + tuple(ctx.ckpts[0].shape), dtype=adj.dtype,
                               device=adj.device)
-            stride = seg[0].numel() * seg.element_size()
         for t0 in reversed(sorted(ctx.ckpts)):
             t1 = min(t0 + k, t_rec)
             asim.restore(ctx.ckpts[t0], t0)
-            lbm.lbm_record_steps(asim.h, t1 - t0, seg.data_ptr(), stride)
-            lbm.lbm_adjoint_sweep(asim.h, seg.data_ptr(), stride, t0, t1 - t0, adj.data_ptr(),
-                                  spare.data_ptr())
+            asim.record(seg[:t1 - t0])
+            asim.sweep(seg[:t1 - t0], t0, adj, spare)
         if 0 in ctx.ckpts:
             asim.restore(ctx.ckpts[0], 0)
         dphi0 = asim.vjp_init(adj, None)
