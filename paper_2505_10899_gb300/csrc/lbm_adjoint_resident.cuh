@@ -136,6 +136,8 @@ __global__ void __launch_bounds__(kAdNT, 1)
     if (at < kAdNX)
       sdesc[at] = make_uint2(tl.slot + (uint32_t)q, (uint32_t)(x + 2) | ((uint32_t)(y + 2) << 10) |
                                                         ((uint32_t)k << 20) | ((uint32_t)side << 23));
+    else
+      atomicOr(run.flags, lbmk::kFlagBounds);  // no plan gives such a tile
   }
   for (int q = tid; q < 12 * (h + 4) + 12 * w; q += kAdNT) {
     int x, y, k, side;
@@ -168,9 +170,11 @@ __global__ void __launch_bounds__(kAdNT, 1)
     if (at < kAdNX)
       rdesc[at] = make_uint2(slot, (uint32_t)(x + 2) | ((uint32_t)(y + 2) << 10) |
                                        ((uint32_t)k << 20) | ((uint32_t)side << 23));
+    else
+      atomicOr(run.flags, lbmk::kFlagBounds);
   }
   __syncthreads();
-  const int nrecv = nrecv_s, nsend = nsend_s;
+  const int nrecv = min(nrecv_s, kAdNX), nsend = min(nsend_s, kAdNX);
 
   // own nodes
   int lx[kAdR], ly[kAdR];
@@ -183,8 +187,9 @@ __global__ void __launch_bounds__(kAdNT, 1)
     ly[r] = act[r] ? k / w : 0;
     lx[r] = act[r] ? k - ly[r] * w : 0;
     const int node = (tl.y0 + ly[r]) * nx + tl.x0 + lx[r];
-    aJx[r] = run.adj[18 * n + node];
-    aJy[r] = run.adj[19 * n + node];
+    const bool ok = LBM_BOUND(run.flags, node, n);
+    aJx[r] = ok ? run.adj[18 * n + node] : R(0);
+    aJy[r] = ok ? run.adj[19 * n + node] : R(0);
   }
   double pacc = 0.0;  // lane q < kNParam: parameter q of this warp
 
@@ -212,7 +217,7 @@ __global__ void __launch_bounds__(kAdNT, 1)
       for (int i = 0; i < 9; ++i) {
         int p;
         const int pos = ad_src(i, x, y, nx, ny, a.walls, &p);
-        G[i] = __ldg(gA + p * n + pos);
+        G[i] = LBM_BOUND(run.flags, pos, n) ? __ldg(gA + p * n + pos) : R(0);
       }
       const R phi = lbmk::sum9(G);
       pq[q] = make_float2(phi, lbmk::psi_of(phi, a.ph.xi));
@@ -231,10 +236,12 @@ __global__ void __launch_bounds__(kAdNT, 1)
       for (int i = 0; i < 9; ++i) {
         int p;
         const int pos = ad_src(i, x, y, nx, ny, a.walls, &p);
-        G[i] = __ldg(gA + p * n + pos);
-        F[i] = __ldg(fA + p * n + pos);
+        const bool ok = LBM_BOUND(run.flags, pos, n);
+        G[i] = ok ? __ldg(gA + p * n + pos) : R(0);
+        F[i] = ok ? __ldg(fA + p * n + pos) : R(0);
       }
-      const R jpx = __ldg(JA + node), jpy = __ldg(JA + n + node);
+      const bool okn = LBM_BOUND(run.flags, node, n);
+      const R jpx = okn ? __ldg(JA + node) : R(0), jpy = okn ? __ldg(JA + n + node) : R(0);
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
         // beyond a wall the ghost row mirrors the wall row
@@ -259,8 +266,8 @@ __global__ void __launch_bounds__(kAdNT, 1)
       if (first) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-          aF[i] = run.adj[i * n + node];
-          aG[i] = run.adj[(9 + i) * n + node];
+          aF[i] = okn ? run.adj[i * n + node] : R(0);
+          aG[i] = okn ? run.adj[(9 + i) * n + node] : R(0);
         }
       } else {
 #pragma unroll
@@ -304,6 +311,7 @@ __global__ void __launch_bounds__(kAdNT, 1)
     const uint32_t set = (j & 1) ? run.nslots : 0u;
     for (int q = tid; q < nsend; q += kAdNT) {
       const uint2 d = sdesc[q];
+      if (!LBM_BOUND(run.flags, d.x, run.nslots)) continue;
       const int x = (int)(d.y & 1023u) - 2, y = (int)((d.y >> 10) & 1023u) - 2;
       const int k = (d.y >> 20) & 7u, side = (d.y >> 23) & 3u;
       int p0, p1, p2;
@@ -332,7 +340,8 @@ __global__ void __launch_bounds__(kAdNT, 1)
         const int row = q / lines, pl_ = row / h;
         const int64_t at = (int64_t)pl_ * n + (tl.y0 + row - pl_ * h) * nx + tl.x0 +
                            min((q - row * lines) * 32, w - 1);
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(st - run.stride + at));
+        if (LBM_BOUND(run.flags, at, 20 * (int64_t)n))
+          asm volatile("prefetch.global.L2 [%0];" ::"l"(st - run.stride + at));
       }
     }
     bool bad = false;
@@ -353,6 +362,7 @@ __global__ void __launch_bounds__(kAdNT, 1)
     for (int q = tid; q < nrecv; q += 2 * kAdNT) {
       const bool two = q + kAdNT < nrecv;
       const uint2 d = rdesc[q], e = two ? rdesc[q + kAdNT] : d;
+      if (!LBM_BOUND(run.flags, d.x, run.nslots) || !LBM_BOUND(run.flags, e.x, run.nslots)) continue;
       R v[3], u[3];
       const uint4 *p = run.slots + set + d.x, *p2 = run.slots + set + e.x;
       bool dv = Word::get(p, v[0], v[1], v[2], tag);
@@ -425,6 +435,7 @@ __global__ void __launch_bounds__(kAdNT, 1)
     if (!act[r]) continue;
     const int y = tl.y0 + ly[r], node = y * nx + tl.x0 + lx[r];
     const bool bt = walls && y == 0, tp = walls && y == ny - 1;
+    if (!LBM_BOUND(run.flags, node, n)) continue;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       run.adj[i * n + node] = pulled(cur, i, 1, lx[r], ly[r], bt, tp);
