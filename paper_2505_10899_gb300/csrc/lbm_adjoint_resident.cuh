@@ -21,10 +21,10 @@
 // around it, and of one the phi adjoint and the populations that move into
 // it: six triples per rim node (k = 0..5 below).
 //
-// Parameter terms: per step and warp as in ad_node (R within a warp); the
-// warp sums accumulate in FP64, lane q of a warp holding parameter q, and
-// enter the CTA's slots in warp order at the end.  They count only if no wait of
-// the sweep gave up (ad_commit).
+// Parameter terms: the sums of a warp's 32 nodes in R, as in ad_node, one per
+// step and node of a thread; they accumulate in FP64, lanes 4q .. 4q+3 of a warp
+// holding parameter q, and enter the CTA's slots in warp order at the end.  They
+// count only if no wait of the sweep gave up (ad_commit).
 //
 // Measured, us per adjoint step (two launches per step -> here): 512 x 256 with
 // walls 23.9 -> 11.6, 384 x 192 21.8 -> 7.8, 201 x 101 with walls 22.6 -> 4.9,
@@ -191,7 +191,8 @@ __global__ void __launch_bounds__(kAdNT, 1)
     aJx[r] = ok ? run.adj[18 * n + node] : R(0);
     aJy[r] = ok ? run.adj[19 * n + node] : R(0);
   }
-  double pacc = 0.0;  // lane q < kNParam: parameter q of this warp
+  static_assert(kNParam <= 8, "a warp's parameter sums");
+  double pacc = 0.0;  // lanes 4q .. 4q+3: parameter q of this warp
 
   // adjoint of the population in plane i (0..8 g, 9..17 f) at own position (x, y)
   auto pulled = [&](const R* L, int i, int f, int x, int y, bool bt, bool tp) -> R {
@@ -224,86 +225,93 @@ __global__ void __launch_bounds__(kAdNT, 1)
     }
     __syncthreads();
     // ---- the reverse arithmetic at the own nodes ------------------------------
-    R gacc[kNParam] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
 #pragma unroll
     for (int r = 0; r < kAdR; ++r) {
-      if (!act[r]) continue;
-      const int x = tl.x0 + lx[r], y = tl.y0 + ly[r], c = lcell(lx[r], ly[r]);
-      const int node = y * nx + x;
-      const bool bt = walls && y == 0, tp = walls && y == ny - 1;
-      R F[9], G[9], Pv[9], Qv[9], aF[9], aG[9];
-#pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        int p;
-        const int pos = ad_src(i, x, y, nx, ny, a.walls, &p);
-        const bool ok = LBM_BOUND(run.flags, pos, n);
-        G[i] = ok ? __ldg(gA + p * n + pos) : R(0);
-        F[i] = ok ? __ldg(fA + p * n + pos) : R(0);
-      }
-      const bool okn = LBM_BOUND(run.flags, node, n);
-      const R jpx = okn ? __ldg(JA + node) : R(0), jpy = okn ? __ldg(JA + n + node) : R(0);
-#pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        // beyond a wall the ghost row mirrors the wall row
-        const int dy = (bt && kAY(i) == -1) || (tp && kAY(i) == 1) ? 0 : kAY(i);
-        const float2 v = pq[c + dy * pl + kAX(i)];
-        Pv[i] = v.x;
-        Qv[i] = v.y;
-      }
-      if (bt || tp) {
-        const R rw = a.rho_g + Pv[0] * a.drho;
-        if (bt) {
-          const R d = rw * a.u_bot * R(1.0 / 6.0);
-          F[5] += d;
-          F[6] -= d;
-        }
-        if (tp) {
-          const R d = rw * a.u_top * R(1.0 / 6.0);
-          F[7] -= d;
-          F[8] += d;
-        }
-      }
-      if (first) {
+      R gacc[kNParam] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
+      if (act[r]) {
+        const int x = tl.x0 + lx[r], y = tl.y0 + ly[r], c = lcell(lx[r], ly[r]);
+        const int node = y * nx + x;
+        const bool bt = walls && y == 0, tp = walls && y == ny - 1;
+        R F[9], G[9], Pv[9], Qv[9], aF[9], aG[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-          aF[i] = okn ? run.adj[i * n + node] : R(0);
-          aG[i] = okn ? run.adj[(9 + i) * n + node] : R(0);
+          int p;
+          const int pos = ad_src(i, x, y, nx, ny, a.walls, &p);
+          const bool ok = LBM_BOUND(run.flags, pos, n);
+          G[i] = ok ? __ldg(gA + p * n + pos) : R(0);
+          F[i] = ok ? __ldg(fA + p * n + pos) : R(0);
         }
-      } else {
+        const bool okn = LBM_BOUND(run.flags, node, n);
+        const R jpx = okn ? __ldg(JA + node) : R(0), jpy = okn ? __ldg(JA + n + node) : R(0);
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-          aF[i] = pulled(cur, i, 1, lx[r], ly[r], bt, tp);
-          aG[i] = pulled(cur, i, 0, lx[r], ly[r], bt, tp);
+          // beyond a wall the ghost row mirrors the wall row
+          const int dy = (bt && kAY(i) == -1) || (tp && kAY(i) == 1) ? 0 : kAY(i);
+          const float2 v = pq[c + dy * pl + kAX(i)];
+          Pv[i] = v.x;
+          Qv[i] = v.y;
+        }
+        if (bt || tp) {
+          const R rw = a.rho_g + Pv[0] * a.drho;
+          if (bt) {
+            const R d = rw * a.u_bot * R(1.0 / 6.0);
+            F[5] += d;
+            F[6] -= d;
+          }
+          if (tp) {
+            const R d = rw * a.u_top * R(1.0 / 6.0);
+            F[7] -= d;
+            F[8] += d;
+          }
+        }
+        if (first) {
+#pragma unroll
+          for (int i = 0; i < 9; ++i) {
+            aF[i] = okn ? run.adj[i * n + node] : R(0);
+            aG[i] = okn ? run.adj[(9 + i) * n + node] : R(0);
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 9; ++i) {
+            aF[i] = pulled(cur, i, 1, lx[r], ly[r], bt, tp);
+            aG[i] = pulled(cur, i, 0, lx[r], ly[r], bt, tp);
+          }
+        }
+        const AdOut<R> o =
+            ad_node_math(a, x, y, F, G, jpx, jpy, Pv, Qv, aF, aG, aJx[r], aJy[r], bt, tp, gacc);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+          nxt[i * kAdL + c] = o.lG[i];
+          nxt[(9 + i) * kAdL + c] = o.lF[i];
+        }
+        const int v = vcell(lx[r], ly[r]);
+        V[v] = o.lgpx;
+        V[kAdV + v] = o.lgpy;
+        V[2 * kAdV + v] = o.llap;
+        V[3 * kAdV + v] = o.lqx;
+        V[4 * kAdV + v] = o.lqy;
+        V[5 * kAdV + v] = R(-10.0 / 3.0) * o.llap + o.lphi;
+        aJx[r] = o.ljpx;
+        aJy[r] = o.ljpy;
+      }
+      // parameter terms: 32 nodes' sums in R, accumulated in FP64.  Every
+      // exchange halves the values a lane holds, so lanes 4q .. 4q+3 end with
+      // parameter q: 9 shuffles for a warp's 8 sums.
+      R sum[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) sum[q] = q < kNParam ? gacc[q < kNParam ? q : 0] : R(0);
+#pragma unroll
+      for (int o = 16, m = 4; m > 0; o >>= 1, m >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int q = 0; q < m; ++q) {
+          const R send = up ? sum[q] : sum[q + m], keep = up ? sum[q + m] : sum[q];
+          sum[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
       }
-      const AdOut<R> o =
-          ad_node_math(a, x, y, F, G, jpx, jpy, Pv, Qv, aF, aG, aJx[r], aJy[r], bt, tp, gacc);
-#pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        nxt[i * kAdL + c] = o.lG[i];
-        nxt[(9 + i) * kAdL + c] = o.lF[i];
-      }
-      const int v = vcell(lx[r], ly[r]);
-      V[v] = o.lgpx;
-      V[kAdV + v] = o.lgpy;
-      V[2 * kAdV + v] = o.llap;
-      V[3 * kAdV + v] = o.lqx;
-      V[4 * kAdV + v] = o.lqy;
-      V[5 * kAdV + v] = R(-10.0 / 3.0) * o.llap + o.lphi;
-      aJx[r] = o.ljpx;
-      aJy[r] = o.ljpy;
-    }
-    // parameter terms: the warp's sums in R, accumulated in FP64
-    {
-      R mine = R(0);
-#pragma unroll
-      for (int q = 0; q < kNParam; ++q) {
-        R v = gacc[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == q) mine = v;
-      }
-      pacc += (double)mine;
+      sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], 2);
+      sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], 1);
+      pacc += (double)sum[0];
     }
     __syncthreads();
     // ---- exchange ---------------------------------------------------------------
@@ -444,7 +452,7 @@ __global__ void __launch_bounds__(kAdNT, 1)
     run.adj[18 * n + node] = aJx[r];
     run.adj[19 * n + node] = aJy[r];
   }
-  if (lane < kNParam) red[warp][lane] = pacc;
+  if ((lane & 3) == 0 && (lane >> 2) < kNParam) red[warp][lane >> 2] = pacc;
   __syncthreads();
   if (tid < kNParam) {
     double v = 0.0;
