@@ -1,5 +1,6 @@
 // FP64 instantiation of the device kernels.
 #define LBM_T double
+#define LBM_PLAIN false
 #include "kern_impl.cuh"
 
 namespace lbmk {

@@ -1,5 +1,7 @@
 // Explicit instantiation of the launch wrappers for precision LBM_T.
-// Included by kern_f32.cu (LBM_T = float) and kern_f64.cu (LBM_T = double).
+// Included by kern_f32.cu (LBM_T = float), kern_f64.cu (LBM_T = double) and, with
+// LBM_PLAIN = true, kern_f64p.cu: the step kernels alone, without the short
+// forms of lbm_math.cuh.
 #include <algorithm>
 #include <type_traits>
 
@@ -12,6 +14,8 @@
 namespace lbmk {
 
 namespace {
+constexpr bool kPlain = LBM_PLAIN;
+
 inline int grid_for(int64_t n, int threads) {
   int64_t b = (n + threads - 1) / threads;
   if (b > 65535 * 8) b = 65535 * 8;
@@ -28,14 +32,14 @@ constexpr int stages_for() {
 template <int BX, bool COUPLED, int MODE>
 cudaError_t step_tma(const StepArgs<LBM_T>& a, int n, cudaStream_t s) {
   using SH = TmaShape<LBM_T, BX, COUPLED, MODE, stages_for<BX>()>;
-  step_kernel_tma<LBM_T, BX, COUPLED, MODE, stages_for<BX>()><<<n, BX, SH::SMEM_BYTES, s>>>(a);
+  step_kernel_tma<LBM_T, BX, COUPLED, MODE, stages_for<BX>(), kPlain><<<n, BX, SH::SMEM_BYTES, s>>>(a);
   return cudaGetLastError();
 }
 
 template <int BX, bool COUPLED, int MODE>
 cudaError_t prep_one() {
   using SH = TmaShape<LBM_T, BX, COUPLED, MODE, stages_for<BX>()>;
-  return cudaFuncSetAttribute(step_kernel_tma<LBM_T, BX, COUPLED, MODE, stages_for<BX>()>,
+  return cudaFuncSetAttribute(step_kernel_tma<LBM_T, BX, COUPLED, MODE, stages_for<BX>(), kPlain>,
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SH::SMEM_BYTES);
 }
 
@@ -63,14 +67,14 @@ cudaError_t step_bx(const StepArgs<LBM_T>& a, bool coupled, int mode, bool tma, 
   } else {
   if (coupled) {
     if (mode == kModeStep)
-      step_kernel<LBM_T, BX, true, kModeStep><<<n, BX, 0, s>>>(a);
+      step_kernel<LBM_T, BX, true, kModeStep, kPlain><<<n, BX, 0, s>>>(a);
     else
-      step_kernel<LBM_T, BX, true, kModeFields><<<n, BX, 0, s>>>(a);
+      step_kernel<LBM_T, BX, true, kModeFields, kPlain><<<n, BX, 0, s>>>(a);
   } else {
     if (mode == kModeStep)
-      step_kernel<LBM_T, BX, false, kModeStep><<<n, BX, 0, s>>>(a);
+      step_kernel<LBM_T, BX, false, kModeStep, kPlain><<<n, BX, 0, s>>>(a);
     else
-      step_kernel<LBM_T, BX, false, kModeFields><<<n, BX, 0, s>>>(a);
+      step_kernel<LBM_T, BX, false, kModeFields, kPlain><<<n, BX, 0, s>>>(a);
   }
   return cudaGetLastError();
   }
@@ -78,16 +82,18 @@ cudaError_t step_bx(const StepArgs<LBM_T>& a, bool coupled, int mode, bool tma, 
 }  // namespace
 
 template <>
-cudaError_t launch_step<LBM_T>(const StepArgs<LBM_T>& a, int bx, bool coupled, int mode,
+cudaError_t launch_step<LBM_T, kPlain>(const StepArgs<LBM_T>& a, int bx, bool coupled, int mode,
                                bool tma, int n_items, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
   switch (bx) {
     case 32: return step_bx<32>(a, coupled, mode, tma, n_items, s);
     case 64: return step_bx<64>(a, coupled, mode, tma, n_items, s);
     case 128: return step_bx<128>(a, coupled, mode, tma, n_items, s);
+#if !LBM_PLAIN  // whole-row widths
     case 96: return step_bx<96>(a, coupled, mode, tma, n_items, s);
     case 192: return step_bx<192>(a, coupled, mode, tma, n_items, s);
     case 256: return step_bx<256>(a, coupled, mode, tma, n_items, s);
+#endif
     default: return cudaErrorInvalidValue;
   }
 }
@@ -95,7 +101,7 @@ cudaError_t launch_step<LBM_T>(const StepArgs<LBM_T>& a, int bx, bool coupled, i
 template <int BX, bool COUPLED>
 cudaError_t persist_bx(const StepArgs<LBM_T>& a, int n_items, int nsteps, int flip,
                        unsigned int* count, unsigned int* gen, cudaStream_t s) {
-  auto kern = step_kernel_persistent<LBM_T, BX, COUPLED>;
+  auto kern = step_kernel_persistent<LBM_T, BX, COUPLED, kPlain>;
   int dev = 0, nsm = 0, per_sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -111,7 +117,7 @@ cudaError_t persist_bx(const StepArgs<LBM_T>& a, int n_items, int nsteps, int fl
 }
 
 template <>
-cudaError_t launch_persistent<LBM_T>(const StepArgs<LBM_T>& a, int bx, bool coupled, int n_items,
+cudaError_t launch_persistent<LBM_T, kPlain>(const StepArgs<LBM_T>& a, int bx, bool coupled, int n_items,
                                      int nsteps, int flip, unsigned int* count,
                                      unsigned int* gen, cudaStream_t s) {
   if (n_items <= 0 || nsteps <= 0) return cudaSuccess;
@@ -132,7 +138,7 @@ struct ResKernel {
   static constexpr size_t BYTES = ResShape<LBM_T, COUPLED, X.pc, X.nx>::SMEM_BYTES;
   static_assert(X.per_sm * (BYTES + 1280) <= 228 * 1024, "shared memory of an SM");
   static const void* fn() {
-    return (const void*)step_resident<LBM_T, COUPLED, X.nt, X.r, X.pc, X.nx, X.per_sm>;
+    return (const void*)step_resident<LBM_T, COUPLED, X.nt, X.r, X.pc, X.nx, X.per_sm, kPlain>;
   }
 };
 
@@ -146,7 +152,7 @@ cudaError_t res_pick(bool coupled, int v, F&& f) {
 }
 
 template <>
-cudaError_t launch_resident<LBM_T>(const StepArgs<LBM_T>& a, bool coupled, int variant,
+cudaError_t launch_resident<LBM_T, kPlain>(const StepArgs<LBM_T>& a, bool coupled, int variant,
                                    const ResTile* tiles, int ntiles, const ResRun& run,
                                    cudaStream_t s) {
   return res_pick(coupled, variant, [&](auto k) {
@@ -159,7 +165,7 @@ cudaError_t launch_resident<LBM_T>(const StepArgs<LBM_T>& a, bool coupled, int v
 }
 
 template <>
-bool resident_fits<LBM_T>(bool coupled, int variant, int ntiles) {
+bool resident_fits<LBM_T, kPlain>(bool coupled, int variant, int ntiles) {
   int dev = 0, nsm = 0, per_sm = 0;
   const cudaError_t e = res_pick(coupled, variant, [&](auto k) -> cudaError_t {
     using KX = decltype(k);
@@ -176,15 +182,19 @@ bool resident_fits<LBM_T>(bool coupled, int variant, int ntiles) {
 }
 
 template <>
-cudaError_t prepare_tma<LBM_T>() {
+cudaError_t prepare_tma<LBM_T, kPlain>() {
   cudaError_t e;
   if ((e = prep_bx<32>()) != cudaSuccess) return e;
   if ((e = prep_bx<64>()) != cudaSuccess) return e;
+#if !LBM_PLAIN
   if ((e = prep_bx<96>()) != cudaSuccess) return e;
   if ((e = prep_bx<192>()) != cudaSuccess) return e;
   if ((e = prep_bx<256>()) != cudaSuccess) return e;
+#endif
   return prep_bx<128>();
 }
+
+#if !LBM_PLAIN
 
 template <>
 size_t tma_smem_bytes<LBM_T>(int bx, bool coupled, int mode) {
@@ -346,5 +356,7 @@ cudaError_t launch_volume_final<LBM_T>(const CaseDev<LBM_T>* cases, const int* c
       cases, case_ids, ncases, part, out, t, toff, slots, stride);
   return cudaGetLastError();
 }
+
+#endif  // !LBM_PLAIN
 
 }  // namespace lbmk

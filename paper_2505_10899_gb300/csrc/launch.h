@@ -15,16 +15,20 @@ inline bool valid_bx(int bx) { return bx == 32 || bx == 64 || bx == 128; }
 // one strip of that width (their own chains, see lbm_api.cu).
 inline bool row_bx(int bx) { return bx == 96 || bx == 192 || bx == 256; }
 
+// PLAIN, here and below: in FP64, the kernels without the short forms of
+// lbm_math.cuh (strips of 32, 64 and 128 columns), which handles with reverse
+// mode run.  A template and not a branch: a launch-uniform branch cost the
+// register kernel its registers (1536 x 1024 with walls 817 -> 906 us per step).
 // tma: use the bulk-copy staged kernel (every case must have nx a multiple
 // of 16 bytes of T and nx >= 4), else the register-pipelined kernel.
-template <typename T>
+template <typename T, bool PLAIN>
 cudaError_t launch_step(const StepArgs<T>& a, int bx, bool coupled, int mode, bool tma,
                         int n_items, cudaStream_t s);
 
 // Persistent register-path kernel (cooperative launch): nsteps steps in one
 // launch; grid = min(n_items, co-resident CTAs).  count/gen: grid-barrier
 // words (zero-initialised, device).
-template <typename T>
+template <typename T, bool PLAIN>
 cudaError_t launch_persistent(const StepArgs<T>& a, int bx, bool coupled, int n_items,
                               int nsteps, int flip, unsigned int* count, unsigned int* gen,
                               cudaStream_t s);
@@ -55,18 +59,18 @@ constexpr ResVariant res_variant(bool f64, bool coupled, int v) {
 }
 
 // Chip-resident kernel (cooperative launch of ntiles CTAs).
-template <typename T>
+template <typename T, bool PLAIN>
 cudaError_t launch_resident(const StepArgs<T>& a, bool coupled, int variant,
                             const ResTile* tiles, int ntiles, const ResRun& run, cudaStream_t s);
 
 // Whether ntiles CTAs of a variant are co-resident on the current device
 // (also allows the variant's dynamic shared memory; before the first launch).
-template <typename T>
+template <typename T, bool PLAIN>
 bool resident_fits(bool coupled, int variant, int ntiles);
 
 // Allow the dynamic shared memory of every TMA kernel variant on the current
 // device (call once per device before the first launch or graph capture).
-template <typename T>
+template <typename T, bool PLAIN>
 cudaError_t prepare_tma();
 
 // Dynamic shared memory of the TMA kernel variant (0 if not available).

@@ -36,7 +36,7 @@
 
 namespace lbmk {
 int set_last_error(int code, const char* msg);
-void drop_graphs(lbm_handle* h);
+int set_plain(lbm_handle* h);
 int synced_valid(lbm_handle* h);
 }  // namespace lbmk
 
@@ -918,11 +918,7 @@ int lbm_adjoint_attach(lbm_handle* h, void* d_scratch, size_t bytes) {
   h->adj_ws_bytes = bytes;
   h->adj_res = lbmk::res_plan_adjoint(h->params[0]);
   h->adj_epoch = 1;
-  if (h->precision == LBM_F64 && !h->pd.plain) {  // see Phys::plain
-    lbmk::drop_graphs(h);                         // captured launches hold the short forms
-    h->pd.plain = 1;
-    h->pd.unit = 0;
-  }
+  if ((rc = lbmk::set_plain(h))) return rc;
   const AdScratch s = carve(h);
   cudaError_t e = cudaMemsetAsync(s.part, 0, (kAdBlocks + 1) * kNParam * sizeof(double),
                                   h->stream);  // partials and accumulator

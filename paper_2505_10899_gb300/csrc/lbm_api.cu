@@ -456,29 +456,58 @@ StepArgs<T> step_args(const lbm_handle* h, int parity, int64_t t_off) {
   return a;
 }
 
-int launch_persist(lbm_handle* h, cudaStream_t s, int parity, int nsteps, int flip) {
+// The launch wrappers of a handle: FP64 handles with reverse mode run the
+// kernels without the short forms (lbm_handle::plain).
+template <typename T>
+cudaError_t step_launch(const lbm_handle* h, const StepArgs<T>& a, int bx, int mode, int n,
+                        cudaStream_t s) {
   const bool coupled = h->flow == LBM_FLOW_COUPLED;
+  if constexpr (sizeof(T) == 8)
+    if (h->plain) return lbmk::launch_step<T, true>(a, bx, coupled, mode, use_tma(h), n, s);
+  return lbmk::launch_step<T, false>(a, bx, coupled, mode, use_tma(h), n, s);
+}
+
+template <typename T>
+cudaError_t persist_launch(lbm_handle* h, int parity, int n, int nsteps, int flip, cudaStream_t s) {
+  const bool coupled = h->flow == LBM_FLOW_COUPLED;
+  const StepArgs<T> a = step_args<T>(h, parity, 0);
+  if constexpr (sizeof(T) == 8)
+    if (h->plain)
+      return lbmk::launch_persistent<T, true>(a, h->tile.bx, coupled, n, nsteps, flip,
+                                              bar_count(h), bar_gen(h), s);
+  return lbmk::launch_persistent<T, false>(a, h->tile.bx, coupled, n, nsteps, flip, bar_count(h),
+                                           bar_gen(h), s);
+}
+
+// Whether the chip-resident kernel of a handle fits the device (and what its
+// staged kernel needs set), asked before the first launch of its kernels.
+template <typename T, bool PLAIN>
+cudaError_t prepare_kernels(lbm_handle* h) {
+  if (h->res.variant >= 0 &&
+      !lbmk::resident_fits<T, PLAIN>(h->flow == LBM_FLOW_COUPLED, h->res.variant,
+                                     (int)h->res.tiles.size()))
+    h->res.variant = -1;
+  // handles without the staged kernel need no attributes of it
+  return h->tma_ok ? lbmk::prepare_tma<T, PLAIN>() : cudaSuccess;
+}
+
+int launch_persist(lbm_handle* h, cudaStream_t s, int parity, int nsteps, int flip) {
   const int n = (int)h->items.size();
   // a launch whose barrier wait gave up leaves arrivals counted: start at 0
   LBM_CUDA(cudaMemsetAsync(bar_count(h), 0, sizeof(unsigned int), s));
-  cudaError_t e;
-  if (h->precision == LBM_F32)
-    e = lbmk::launch_persistent<float>(step_args<float>(h, parity, 0), h->tile.bx, coupled, n,
-                                       nsteps, flip, bar_count(h), bar_gen(h), s);
-  else
-    e = lbmk::launch_persistent<double>(step_args<double>(h, parity, 0), h->tile.bx, coupled, n,
-                                        nsteps, flip, bar_count(h), bar_gen(h), s);
+  const cudaError_t e = h->precision == LBM_F32 ? persist_launch<float>(h, parity, n, nsteps, flip, s)
+                                                : persist_launch<double>(h, parity, n, nsteps, flip, s);
   if (e != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("persistent launch: ") + cudaGetErrorString(e));
   return LBM_OK;
 }
 
 // Whether the chip-resident kernel may run this handle's steps at all.  A
-// handle with reverse mode in FP64 (Phys::plain) takes it only where the
+// handle with reverse mode in FP64 (lbm_handle::plain) takes it only where the
 // single steps run the staged kernel, whose bits it gives; the register
 // kernel contracts some multiply-adds differently, and the parameter
 // derivatives of a state that differs in its last bits differ by 1e-9.
 bool res_allowed(const lbm_handle* h) {
-  return h->res.variant >= 0 && (!h->pd.plain || h->tma_ok);
+  return h->res.variant >= 0 && (!h->plain || h->tma_ok);
 }
 
 // Whether long runs take it now: no other kernel was asked for or measured
@@ -520,9 +549,16 @@ int launch_res(lbm_handle* h, int nsteps, int store, void* rec, int64_t stride) 
   r.rec = rec;
   r.rec_stride = stride / (int64_t)sizeof(T);
   h->res_epoch += (uint32_t)nsteps;
-  const cudaError_t e = lbmk::launch_resident<T>(
-      step_args<T>(h, h->parity, 0), h->flow == LBM_FLOW_COUPLED, h->res.variant,
-      (const lbmk::ResTile*)(h->ws + h->L.rtiles), (int)h->res.tiles.size(), r, h->stream);
+  const StepArgs<T> a = step_args<T>(h, h->parity, 0);
+  const bool coupled = h->flow == LBM_FLOW_COUPLED;
+  const auto* tiles = (const lbmk::ResTile*)(h->ws + h->L.rtiles);
+  const int nt = (int)h->res.tiles.size();
+  cudaError_t e = cudaSuccess;
+  bool done = false;
+  if constexpr (sizeof(T) == 8)
+    if ((done = h->plain))
+      e = lbmk::launch_resident<T, true>(a, coupled, h->res.variant, tiles, nt, r, h->stream);
+  if (!done) e = lbmk::launch_resident<T, false>(a, coupled, h->res.variant, tiles, nt, r, h->stream);
   if (e != cudaSuccess)
     return fail(LBM_ERR_CUDA, std::string("resident launch: ") + cudaGetErrorString(e));
   return LBM_OK;
@@ -570,7 +606,7 @@ int enqueue_steps(lbm_handle* h, cudaStream_t s, int parity, int count, bool fli
         StepArgs<float> a = step_args<float>(h, par, toff);
         a.items = h->items_dev + i0;
         a.vol_part = (vol && h->track) ? h->part + (int64_t)i0 * lbmk::kMaxRegions : nullptr;
-        e = lbmk::launch_step<float>(a, bx, coupled, lbmk::kModeStep, use_tma(h), ni, sc);
+        e = step_launch<float>(h, a, bx, lbmk::kModeStep, ni, sc);
         if (e == cudaSuccess && vol && h->track)
           e = lbmk::launch_volume_final<float>((const CaseDev<float>*)h->cases_dev,
                                                h->chain_cases_dev + q0, nc, h->part, h->track,
@@ -580,7 +616,7 @@ int enqueue_steps(lbm_handle* h, cudaStream_t s, int parity, int count, bool fli
         StepArgs<double> a = step_args<double>(h, par, toff);
         a.items = h->items_dev + i0;
         a.vol_part = (vol && h->track) ? h->part + (int64_t)i0 * lbmk::kMaxRegions : nullptr;
-        e = lbmk::launch_step<double>(a, bx, coupled, lbmk::kModeStep, use_tma(h), ni, sc);
+        e = step_launch<double>(h, a, bx, lbmk::kModeStep, ni, sc);
         if (e == cudaSuccess && vol && h->track)
           e = lbmk::launch_volume_final<double>((const CaseDev<double>*)h->cases_dev,
                                                h->chain_cases_dev + q0, nc, h->part, h->track,
@@ -751,9 +787,8 @@ int do_fields(lbm_handle* h, int c, double* phi, double* ux, double* uy, double*
   a.out_ux = st + n;
   a.out_uy = st + 2 * n;
   a.out_p = st + 3 * n;
-  cudaError_t e = lbmk::launch_step<T>(a, h->chain_bx[h->case_chain[c]], h->flow == LBM_FLOW_COUPLED,
-                                       lbmk::kModeFields, use_tma(h),
-                                       h->item_end[c] - h->item_begin[c], h->stream);
+  cudaError_t e = step_launch<T>(h, a, h->chain_bx[h->case_chain[c]], lbmk::kModeFields,
+                                 h->item_end[c] - h->item_begin[c], h->stream);
   if (e != cudaSuccess) return fail(LBM_ERR_CUDA, std::string("fields: ") + cudaGetErrorString(e));
   double* outs[4] = {phi, ux, uy, p};
   for (int q = 0; q < 4; ++q)
@@ -896,7 +931,15 @@ int retile(lbm_handle* h, const Tiling& t, int nchains) {
 
 namespace lbmk {
 int set_last_error(int code, const char* msg) { return fail(code, msg); }
-void drop_graphs(lbm_handle* h) { drop_graph(h); }
+// From here on the handle steps by the kernels without the short forms.
+int set_plain(lbm_handle* h) {
+  if (h->precision != LBM_F64 || h->plain) return LBM_OK;
+  drop_graph(h);  // captured launches are of the others
+  const cudaError_t e = prepare_kernels<double, true>(h);
+  if (e != cudaSuccess) return fail(LBM_ERR_CUDA, cudaGetErrorString(e));
+  h->plain = true;
+  return LBM_OK;
+}
 int synced_valid(lbm_handle* h) { return sync_valid(h); }
 }  // namespace lbmk
 
@@ -1002,25 +1045,20 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace, size_t 
     if (cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming) != cudaSuccess)
       return cleanup(fail(LBM_ERR_CUDA, "cannot create chain events"));
   }
-  if (h->tma_ok) {  // handles without the staged kernel need no attributes of it
-    cudaError_t e = h->precision == LBM_F32 ? lbmk::prepare_tma<float>() : lbmk::prepare_tma<double>();
+  {
+    cudaError_t e = h->precision == LBM_F32 ? prepare_kernels<float, false>(h)
+                                            : prepare_kernels<double, false>(h);
     if (e != cudaSuccess)
       return cleanup(fail(LBM_ERR_CUDA, std::string("kernel attributes: ") + cudaGetErrorString(e)));
   }
   if (cudaMemsetAsync(h->ws + h->L.hdr, 0, 64, h->stream) != cudaSuccess)
     return cleanup(fail(LBM_ERR_CUDA, "header upload failed"));
-  if (h->res.variant >= 0) {
-    const bool coupled = h->flow == LBM_FLOW_COUPLED;
-    const int nt = (int)h->res.tiles.size();
-    if (!(h->precision == LBM_F32 ? lbmk::resident_fits<float>(coupled, h->res.variant, nt)
-                                  : lbmk::resident_fits<double>(coupled, h->res.variant, nt)))
-      h->res.variant = -1;
-    else if (cudaMemcpyAsync(h->ws + h->L.rtiles, h->res.tiles.data(),
-                             nt * sizeof(lbmk::ResTile), cudaMemcpyHostToDevice,
-                             h->stream) != cudaSuccess ||
-             cudaMemsetAsync(h->ws + h->L.rslots, 0, h->L.rslot_bytes, h->stream) != cudaSuccess)
-      return cleanup(fail(LBM_ERR_CUDA, "tile upload failed"));
-  }
+  if (h->res.variant >= 0 &&
+      (cudaMemcpyAsync(h->ws + h->L.rtiles, h->res.tiles.data(),
+                       h->res.tiles.size() * sizeof(lbmk::ResTile), cudaMemcpyHostToDevice,
+                       h->stream) != cudaSuccess ||
+       cudaMemsetAsync(h->ws + h->L.rslots, 0, h->L.rslot_bytes, h->stream) != cudaSuccess))
+    return cleanup(fail(LBM_ERR_CUDA, "tile upload failed"));
   // items, chains and cases; labels planes: zero (region 0 everywhere)
   // until lbm_set_regions
   rc = upload_plan(h);

@@ -97,6 +97,9 @@ struct lbm_handle {
   bool res_auto = true;
   int res_min = lbmk::kResMinSteps;
   uint32_t res_epoch = 1;
+  // FP64 handle with reverse mode: division, root, logarithm and the general
+  // collision in place of their short forms (lbm_math.cuh)
+  bool plain = false;
   // reverse mode (lbm_adjoint_attach): caller-provided FP64 scratch
   char* adj_ws = nullptr;
   size_t adj_ws_bytes = 0;

@@ -129,8 +129,9 @@ __device__ __forceinline__ void write_volume_partial(double vacc, double* vred, 
 // ---------------------------------------------------------------------------
 //   COUPLED: f and g (true) or g only with the prescribed vortex (false).
 //   MODE:    kModeStep collides and stores; kModeFields writes phi, u, p.
+//   PLAIN:   FP64 without the short forms of lbm_math.cuh.
 // ---------------------------------------------------------------------------
-template <typename T, int BX, bool COUPLED, int MODE, bool COHERENT>
+template <typename T, int BX, bool COUPLED, int MODE, bool COHERENT, bool PLAIN>
 __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T, BX>& ring,
                                           double* vred) {
   const Item it = a.items[item];
@@ -171,6 +172,7 @@ __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T
   const int hcm = (hc == 0) ? nx - 1 : hc - 1;
   const int hcp = (hc == nx - 1) ? 0 : hc + 1;
 
+  const T xi = a.ph.xi;
   const bool do_vol = (MODE == kModeStep) && (a.vol_part != nullptr);
   double vacc = 0.0;
   CaseK<T> K = case_consts<T, COUPLED>(a, cdp, xc);
@@ -242,11 +244,11 @@ __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T
     const int s = (k + 4) & 3;
     if (act) {
       const T phi = sum9(G);
-      ring.put(s, tid + 1, phi, psi_of(phi, a.ph));
+      ring.put(s, tid + 1, phi, step_psi<PLAIN>(phi, xi));
     }
     if (hthr) {
       const T phi = sum9(H);
-      ring.put(s, hslot, phi, psi_of(phi, a.ph));
+      ring.put(s, hslot, phi, step_psi<PLAIN>(phi, xi));
     }
   };
 
@@ -290,7 +292,7 @@ __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T
                       cdp->u_top);
       if (!COUPLED) vortex_row(K, y);
       const NodeOut<T> o =
-          node_update<T, COUPLED, MODE>(a.ph, K, C.F, C.G, C.lo, C.J[0], C.J[1], S);
+          node_update<T, COUPLED, MODE, PLAIN>(a.ph, K, C.F, C.G, C.lo, C.J[0], C.J[1], S);
       const uint32_t node = rowoff(y) + (uint32_t)xc;
       if (MODE == kModeStep) {
         store_node<T, COUPLED>(fd, gd, Jd, lod, P, node, C.F, C.G, C.lo, o, a.flags, nn);
@@ -316,11 +318,11 @@ __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T
   __syncthreads();  // the ring is reused by the next item of a persistent CTA
 }
 
-template <typename T, int BX, bool COUPLED, int MODE>
+template <typename T, int BX, bool COUPLED, int MODE, bool PLAIN>
 __global__ void __launch_bounds__(BX) step_kernel(const StepArgs<T> a) {
   __shared__ Ring<T, BX> ring;
   __shared__ double vred[BX / 32];
-  step_item<T, BX, COUPLED, MODE, false>(a, blockIdx.x, ring, vred);
+  step_item<T, BX, COUPLED, MODE, false, PLAIN>(a, blockIdx.x, ring, vred);
 }
 
 // ---------------------------------------------------------------------------
@@ -369,7 +371,7 @@ __device__ __forceinline__ bool grid_barrier(const GridBar& b, int32_t* flags,
   return ok_s != 0;
 }
 
-template <typename T, int BX, bool COUPLED>
+template <typename T, int BX, bool COUPLED, bool PLAIN>
 __global__ void __launch_bounds__(BX) step_kernel_persistent(const StepArgs<T> a, int n_items,
                                                              int nsteps, int flip, GridBar bar) {
   __shared__ Ring<T, BX> ring;
@@ -381,7 +383,7 @@ __global__ void __launch_bounds__(BX) step_kernel_persistent(const StepArgs<T> a
       as.t_off = a.t_off + s;
     }
     for (int item = blockIdx.x; item < n_items; item += gridDim.x)
-      step_item<T, BX, COUPLED, kModeStep, true>(as, item, ring, vred);
+      step_item<T, BX, COUPLED, kModeStep, true, PLAIN>(as, item, ring, vred);
     if (s + 1 < nsteps && !grid_barrier(bar, a.flags, a.wait_cycles)) return;
   }
 }

@@ -63,7 +63,7 @@ struct TmaShape {
 // The kernel body, for strips that hold a whole row (FROW: x0 = 0 and
 // nx <= BX) or not; the kernel picks one per CTA, so that the strips of wide
 // rows keep compile-time staged positions.
-template <typename T, int BX, bool COUPLED, int MODE, int S, bool FROW>
+template <typename T, int BX, bool COUPLED, int MODE, int S, bool FROW, bool PLAIN>
 __device__ __forceinline__ void tma_body(const StepArgs<T>& a, uint4* const rows) {
   using SH = TmaShape<T, BX, COUPLED, MODE, S>;
   constexpr int SEG = SH::SEG, NPL = SH::NPL, NJ = SH::NJ, STAGE = SH::STAGE;
@@ -114,6 +114,7 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a, uint4* const rows
   const int om = spos(tid, -1), o0 = spos(tid, 0), op = spos(tid, 1);
   const int hm = spos(hcol, -1), h0 = spos(hcol, 0), hp = spos(hcol, 1);
 
+  const T xi = a.ph.xi;
   const bool do_vol = (MODE == kModeStep) && (a.vol_part != nullptr);
   double vacc = 0.0;
   CaseK<T> K = case_consts<T, COUPLED>(a, cdp, xc);
@@ -211,12 +212,12 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a, uint4* const rows
     if (act) {
       staged_g(st, om, o0, op, G);
       const T phi = sum9(G);
-      ring.put(s, tid + 1, phi, psi_of(phi, a.ph));
+      ring.put(s, tid + 1, phi, step_psi<PLAIN>(phi, xi));
     }
     if (hthr) {
       staged_g(st, hm, h0, hp, G);
       const T phi = sum9(G);
-      ring.put(s, hslot, phi, psi_of(phi, a.ph));
+      ring.put(s, hslot, phi, step_psi<PLAIN>(phi, xi));
     }
   };
 
@@ -292,7 +293,7 @@ __device__ __forceinline__ void tma_body(const StepArgs<T>& a, uint4* const rows
       // node, is left out here; lbm_volume counts it)
       if (do_vol) vacc += (double)Sn.p;
       if (!COUPLED) vortex_row(K, y);
-      const NodeOut<T> o = node_update<T, COUPLED, MODE>(a.ph, K, F, G, glo, jpx, jpy, Sn);
+      const NodeOut<T> o = node_update<T, COUPLED, MODE, PLAIN>(a.ph, K, F, G, glo, jpx, jpy, Sn);
       if (MODE == kModeStep) {
         store_node<T, COUPLED>(fd, gd, Jd, lod, P, node, F, G, glo, o, a.flags,
                                (uint32_t)nx * (uint32_t)ny);
@@ -330,16 +331,16 @@ constexpr int tma_min_blocks() {
                         : 1;
 }
 
-template <typename T, int BX, bool COUPLED, int MODE, int S>
+template <typename T, int BX, bool COUPLED, int MODE, int S, bool PLAIN>
 __global__ void __launch_bounds__(BX, (tma_min_blocks<T, BX>()))
     step_kernel_tma(const StepArgs<T> a) {
   using SH = TmaShape<T, BX, COUPLED, MODE, S>;
   __shared__ uint4 rows[SH::NPL + SH::NJ + SH::NPAD];
   const Item it = a.items[blockIdx.x];
   if (it.x0 == 0 && a.cases[it.c].nx <= BX)
-    tma_body<T, BX, COUPLED, MODE, S, true>(a, rows);
+    tma_body<T, BX, COUPLED, MODE, S, true, PLAIN>(a, rows);
   else
-    tma_body<T, BX, COUPLED, MODE, S, false>(a, rows);
+    tma_body<T, BX, COUPLED, MODE, S, false, PLAIN>(a, rows);
 }
 
 }  // namespace lbmk

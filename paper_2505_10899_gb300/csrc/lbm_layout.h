@@ -65,7 +65,6 @@ struct Phys {
   T gsD[kQ], ghD3[kQ];  // ghD3 = ghD / 3 (the source moments carry a 1/3)
   double vU, vT;        // prescribed vortex amplitude and period
   int32_t unit;         // all free rates are 1 (FP64 takes a shorter collision)
-  int32_t plain;        // FP64 by division, root and logarithm, general collision: reverse mode
 };
 
 struct Item {

@@ -5,7 +5,7 @@
 // by a square root (about 17) and a division and a logarithm (about 36).
 // With the short collision of lbm_node.cuh: 64 uneven FP64 cases 3.39 -> 2.21
 // ms per step.  The reverse mode and the steps of handles that have it attached
-// take the division, root and logarithm (Phys::plain): d psi/d phi reaches 1e10,
+// take the division, root and logarithm (lbm_handle::plain): d psi/d phi reaches 1e10,
 // and the derivatives of a run move by up to 1e-8 with its states' last bits.
 //   rcp, rsq: the hardware's approximation (PTX rcp/rsqrt.approx.ftz.f64, 20
 //   bits) and one third-order Newton step: with e = 1 - x y, 1/x = y (1 + e +

@@ -87,26 +87,25 @@ __device__ __forceinline__ T psi_of(T phi, T xi) {
 }
 
 // The same, a reciprocal and a reciprocal square root in the forward step: in
-// FP64 the short forms of lbm_math.cuh, unless the handle asks for the division,
-// root and logarithm of Num<double> (Phys::plain, a launch-uniform branch: 64
-// uneven FP64 cases, 8 steps 18.16 ms without it, 17.90 with it).
-template <typename T>
-__device__ __forceinline__ T psi_of(T phi, const Phys<T>& ph) {
-  if constexpr (sizeof(T) == 8) {
-    const T pc = Num<T>::clamp01(phi), a = pc + ph.xi, b = (T(1) - pc) + ph.xi;
-    return ph.plain ? Num<T>::lratio(a, b) : lratio64(a, b);
+// FP64 the short forms of lbm_math.cuh, or (PLAIN) the division, root and
+// logarithm of Num<double>.
+template <bool PLAIN, typename T>
+__device__ __forceinline__ T step_psi(T phi, T xi) {
+  if constexpr (sizeof(T) == 8 && !PLAIN) {
+    const T pc = Num<T>::clamp01(phi);
+    return lratio64(pc + xi, (T(1) - pc) + xi);
   } else {
-    return psi_of(phi, ph.xi);
+    return psi_of(phi, xi);
   }
 }
-template <typename T>
-__device__ __forceinline__ T step_rcp(T x, const Phys<T>& ph) {
-  if constexpr (sizeof(T) == 8) return ph.plain ? Num<T>::rcp(x) : rcp64(x);
+template <bool PLAIN, typename T>
+__device__ __forceinline__ T step_rcp(T x) {
+  if constexpr (sizeof(T) == 8 && !PLAIN) return rcp64(x);
   else return Num<T>::rcp(x);
 }
-template <typename T>
-__device__ __forceinline__ T step_rsq(T x, const Phys<T>& ph) {
-  if constexpr (sizeof(T) == 8) return ph.plain ? Num<T>::rsq(x) : rsq64(x);
+template <bool PLAIN, typename T>
+__device__ __forceinline__ T step_rsq(T x) {
+  if constexpr (sizeof(T) == 8 && !PLAIN) return rsq64(x);
   else return Num<T>::rsq(x);
 }
 
@@ -343,7 +342,7 @@ __device__ __forceinline__ void g_unit(const Phys<double>& ph, double (&G)[9], d
   G[0] = phi - (((G[1] + G[2]) + (G[3] + G[4])) + ((G[5] + G[6]) + (G[7] + G[8])));
 }
 
-template <typename T, bool COUPLED, int MODE>
+template <typename T, bool COUPLED, int MODE, bool PLAIN>
 __device__ __forceinline__ NodeOut<T> node_update(const Phys<T>& ph, const CaseK<T>& K,
                                                   T (&Fc)[9], T (&Gc)[9], T& Glo, T jpx,
                                                   T jpy, const Stencil<T>& S) {
@@ -367,8 +366,8 @@ __device__ __forceinline__ NodeOut<T> node_update(const Phys<T>& ph, const CaseK
   bool unit = false;  // FP64 with unit free rates: the short collision
   if (COUPLED) {
     const T rho = K.rho_g + phi * K.drho;  // linear rho(phi)
-    const T irho = step_rcp(rho, ph);
-    if constexpr (sizeof(T) == 8) {
+    const T irho = step_rcp<PLAIN>(rho);
+    if constexpr (sizeof(T) == 8 && !PLAIN) {
       if (ph.unit) {
         f_unit<MODE>(K, Fc, phi, rho, irho, gpx, gpy, Fx, Fy, o);
         unit = true;
@@ -399,7 +398,7 @@ __device__ __forceinline__ NodeOut<T> node_update(const Phys<T>& ph, const CaseK
       if (K.var_tau) {
         const T mu_v = K.mu_g + phi * K.dmu;
         const T tau = T(3) * mu_v * irho + T(0.5);  // Eq. 27
-        const T s7 = step_rcp(tau, ph);
+        const T s7 = step_rcp<PLAIN>(tau);
         sD7 = T(-0.25) * s7;
         hD7 = T(0.25) - T(0.125) * s7;
       }
@@ -430,13 +429,13 @@ __device__ __forceinline__ NodeOut<T> node_update(const Phys<T>& ph, const CaseK
     const T pc = Num<T>::clamp01(phi);
     const T ta = pc + ph.xi, tb = (T(1) - pc) + ph.xi;
     const T q2 = qx * qx + qy * qy;
-    const T iq = (q2 >= ph.qmin2) ? step_rsq(q2, ph) : T(0);  // n := 0 on ridges of psi
+    const T iq = (q2 >= ph.qmin2) ? step_rsq<PLAIN>(q2) : T(0);  // n := 0 on ridges of psi
     // (lambda/W) [1 - tanh^2(2psi/W)] / |grad psi|, tanh via Eqs. 13-15
     const T sh = ph.lamW * ph.tfac * ta * tb * iq;
     const T Vx = T(3) * dJx + sh * qx;  // d_t(phi u)/c_s^2 + sharpening flux
     const T Vy = T(3) * dJy + sh * qy;
     const T Lam = mu + ph.lambda * phi;
-    if constexpr (sizeof(T) == 8) {
+    if constexpr (sizeof(T) == 8 && !PLAIN) {
       if (ph.unit) {
         g_unit(ph, Gc, phi, Lam, Jx, Jy, Vx, Vy);
         return o;

@@ -39,7 +39,7 @@
 // Per step: collide (shared -> shared), barrier, send the rim, form phi and
 // psi of the nodes whose pull needs no rim, receive the rim, barrier, phi and
 // psi of the remaining nodes, barrier.  The per-node arithmetic is that of
-// the other step kernels (sum9, psi_of, node_update).
+// the other step kernels (sum9, step_psi, node_update).
 //
 // Every wait is bounded (StepArgs::wait_cycles); on expiry the CTA raises
 // kFlagTimeout and returns, and so do its neighbours in turn.  No asynchronous
@@ -130,7 +130,7 @@ __device__ __forceinline__ uint32_t res_desc(int cell, int p0, int p1, int p2) {
   return (uint32_t)cell | ((uint32_t)p0 << 12) | ((uint32_t)p1 << 17) | ((uint32_t)p2 << 22);
 }
 
-template <typename T, bool COUPLED, int NT, int R, int PC, int NX, int MINB>
+template <typename T, bool COUPLED, int NT, int R, int PC, int NX, int MINB, bool PLAIN>
 __global__ void __launch_bounds__(NT, MINB)
     step_resident(const StepArgs<T> a, const ResTile* __restrict__ tiles, const ResRun run) {
   using SH = ResShape<T, COUPLED, PC, NX>;
@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(NT, MINB)
   const uint32_t P = (uint32_t)cdp->plane, nn = (uint32_t)nx * (uint32_t)ny;
   const bool walls = cdp->walls != 0;
   const bool wbot = walls && tl.y0 == 0, wtop = walls && tl.y0 + h == ny;
+  const T xi = a.ph.xi;
   auto cell_of = [&](int x, int y) -> int { return (y + 2) * pw + x + 2; };
 
   const T* gs = cdp->g[a.parity];
@@ -346,7 +347,7 @@ __global__ void __launch_bounds__(NT, MINB)
     const T phi = sum9(G);
     typename Pair<T>::type v;
     v.x = phi;
-    v.y = psi_of(phi, a.ph);
+    v.y = step_psi<PLAIN>(phi, xi);
     pq[dst] = v;
   };
   // own nodes away from the tile's edge: no rim needed
@@ -423,7 +424,7 @@ __global__ void __launch_bounds__(NT, MINB)
         K.sy2 = sy2[r];
       }
       const NodeOut<T> o =
-          node_update<T, COUPLED, kModeStep>(a.ph, K, F, G, lo[r], jx[r], jy[r], S);
+          node_update<T, COUPLED, kModeStep, PLAIN>(a.ph, K, F, G, lo[r], jx[r], jy[r], S);
       jx[r] = o.Jx;
       jy[r] = o.Jy;
 #pragma unroll

@@ -2,8 +2,8 @@
 
 d psi / d phi is up to 1/xi = 1e10 in the bulk, so the derivatives of a run move by up to 1e-8 when
 the last bits of its states do.  A handle with reverse mode attached therefore steps by division,
-root and logarithm and the general collision (Phys::plain), and every route to a state gives the
-bits of the single-step kernel.
+root and logarithm and the general collision (lbm_handle::plain), and every route to a state gives
+the bits of the single-step kernel.
 
 The recorded values are those of the library before its FP64 step had shorter forms (reciprocal and
 logarithm of lbm_math.cuh, collision at unit rates).  The runs below are among those that show a
