@@ -955,8 +955,9 @@ def adjoint_sweep_timing(dev, precisions=("f32", "f64"), nrec=256):
     """Reverse-mode step against the forward step on the sheared droplet in
     a 512 x 256 channel (walls at -U and +U = 0.01, R = 40, Ca = 0.1,
     Re = 0.1), per precision: the forward step autotuned and replayed from
-    graphs, then lbm_record_steps of nrec states and one lbm_adjoint_sweep
-    over them (two launches per step), both timed with CUDA events."""
+    graphs or run on the chip, then lbm_record_steps of nrec states and one
+    lbm_adjoint_sweep over them (one launch where the grid fits the chip in
+    FP32, else two per step), both timed with CUDA events."""
     import torch
     from paper_2505_10899_gb300 import adjoint as A
     from paper_2505_10899_gb300 import lbm

@@ -132,8 +132,8 @@ int lbm3_get_tiling(const lbm3_handle* h, int32_t* bx, int32_t* by, int32_t* zc,
 /* Step-kernel variant.  All variants solve the same equations (variants 5 and
  * 6 in a shorter form: equal up to rounding).
  *   0: automatic -- the register kernel until lbm3_autotune picks the
- *      fastest (on a tile the register kernel does not run, with the
- *      default tile (32, 8));
+ *      fastest (lbm3_init starts on the tile (32, 4); selected on a tile that
+ *      the register kernel does not run, (32, 8));
  *   1: register-pipelined loads (any precision; tiles of variants 1-3,
  *      others switch to (32, 8));
  *   2 / 3: asynchronous 4-byte copies (cp.async) through shared memory,
@@ -161,7 +161,7 @@ int lbm3_get_tiling(const lbm3_handle* h, int32_t* bx, int32_t* by, int32_t* zc,
 int lbm3_set_kernel(lbm3_handle* h, int32_t variant);
 int32_t lbm3_get_kernel(const lbm3_handle* h);
 
-/* Bound of the device waits of the bulk-copy variants (4 to 6), in SM clock
+/* Bound of the device waits of the staged variants (4 to 6), in SM clock
  * cycles: the waits for their staged planes.  A wait that gives up makes
  * lbm3_status report LBM_ERR_TIMEOUT; the CTA first waits, with the default
  * bound, for the copies it issued, then returns, and the step's results are

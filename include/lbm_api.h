@@ -142,7 +142,8 @@ int lbm_init(const lbm_params* cases, int32_t ncases, void* d_workspace,
  * d_t(phi u) by backward difference.  Asynchronous on the handle's stream.
  * Batches that fit the SMs' shared memory (about 150,000 nodes in FP32,
  * 75,000 in FP64) run 4 steps or more as cooperative launches of up to 1,024
- * steps that keep the state on the chip, unless another kernel was asked for,
+ * steps that keep the state on the chip, unless another kernel was asked for
+ * or measured faster (lbm_autotune, which also sets from how many steps on),
  * volumes are tracked or the stream is being captured.  Otherwise
  * runs of 4 steps or more are cut into chunks of up to 64 steps; the first
  * chunk of a given length (and source buffer) is launched directly, and
@@ -259,12 +260,12 @@ int lbm_set_tiling(lbm_handle* h, int32_t bx, int32_t rows);
  * Where the batch fits the chip-resident kernel (see lbm_step) that is timed
  * too, and kept or left for longer runs (from 1 to 4 steps on, as measured)
  * beside the fastest of variants 1 and 2, which serves the others (shorter runs,
- * tracked volumes, captured streams) and is what best_kernel, best_bx, best_rows and lbm_get_kernel report; best_ms is
- * the fastest of all, and lbm_get_resident says which it was.  Elsewhere variant
- * 3 is timed as one persistent launch, unless volumes are tracked.  Trial
- * launches read the current state and write only the buffers the next step
- * overwrites, so the state, the step index and the error flags do not change.
- * Outputs may be NULL.  Synchronises. */
+ * tracked volumes, captured streams) and is what best_kernel, best_bx, best_rows
+ * and lbm_get_kernel report; best_ms is the fastest of all, and lbm_get_resident
+ * says which it was.  Elsewhere variant 3 is timed as one persistent launch,
+ * unless volumes are tracked.  Trial launches read the current state and write
+ * only the buffers the next step overwrites, so the state, the step index and
+ * the error flags do not change.  Outputs may be NULL.  Synchronises. */
 int lbm_autotune(lbm_handle* h, int32_t trials, int32_t* best_kernel,
                  int32_t* best_bx, int32_t* best_rows, double* best_ms);
 

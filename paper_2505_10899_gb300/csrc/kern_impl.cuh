@@ -63,7 +63,7 @@ cudaError_t step_bx(const StepArgs<LBM_T>& a, bool coupled, int mode, bool tma, 
                              : step_tma<BX, false, kModeFields>(a, n, s);
   }
   if constexpr (BX != 32 && BX != 64 && BX != 128) {
-    return cudaErrorInvalidValue;  // whole-row widths: bulk-copy kernel only
+    return cudaErrorInvalidValue;  // whole-row widths: staged kernel only
   } else {
   if (coupled) {
     if (mode == kModeStep)

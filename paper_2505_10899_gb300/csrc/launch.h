@@ -11,7 +11,7 @@ namespace lbmk {
 // Strip widths of a tiling (threads per CTA of the step kernels).
 inline bool valid_bx(int bx) { return bx == 32 || bx == 64 || bx == 128; }
 
-// Strip widths the bulk-copy kernel also runs, for cases whose whole row is
+// Strip widths the staged kernel also runs, for cases whose whole row is
 // one strip of that width (their own chains, see lbm_api.cu).
 inline bool row_bx(int bx) { return bx == 96 || bx == 192 || bx == 256; }
 
@@ -19,7 +19,7 @@ inline bool row_bx(int bx) { return bx == 96 || bx == 192 || bx == 256; }
 // lbm_math.cuh (strips of 32, 64 and 128 columns), which handles with reverse
 // mode run.  A template and not a branch: a launch-uniform branch cost the
 // register kernel its registers (1536 x 1024 with walls 817 -> 906 us per step).
-// tma: use the bulk-copy staged kernel (every case must have nx a multiple
+// tma: use the staged kernel (every case must have nx a multiple
 // of 16 bytes of T and nx >= 4), else the register-pipelined kernel.
 template <typename T, bool PLAIN>
 cudaError_t launch_step(const StepArgs<T>& a, int bx, bool coupled, int mode, bool tma,

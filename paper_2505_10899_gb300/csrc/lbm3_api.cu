@@ -452,7 +452,8 @@ int lbm3_set_kernel(lbm3_handle* h, int32_t variant) {
   int bx = h->bx, by = h->by;
   const int v = variant ? variant : lbmk3::kVarRegs;
   if (v == lbmk3::kVarRegs && !lbmk3::tile_regs_ok(bx, by)) {
-    // automatic or register kernel on a tile it does not run: the default tile
+    // automatic or register kernel on a tile it does not run: the documented
+    // fallback (lbm3_init's own default, 32 x 4, is the faster one)
     bx = 32;
     by = 8;
   }

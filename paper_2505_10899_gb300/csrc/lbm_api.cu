@@ -1242,7 +1242,7 @@ int lbm_set_kernel(lbm_handle* h, int32_t variant) {
   if (!h) return fail(LBM_ERR_ARG, "null handle");
   if (variant < 0 || variant > 3) return fail(LBM_ERR_ARG, "kernel variant must be 0, 1, 2 or 3");
   if (variant == 2 && !h->tma_ok)
-    return fail(LBM_ERR_ARG, "bulk-copy kernel needs nx a multiple of 16 bytes and nx >= 4");
+    return fail(LBM_ERR_ARG, "staged kernel needs nx a multiple of 16 bytes and nx >= 4");
   if (variant == 3 && total_nodes(h) > kPersistMaxNodes)
     return fail(LBM_ERR_ARG, "persistent kernel is for batches of at most 4 Mi nodes");
   if (variant != h->kernel) {

@@ -78,8 +78,8 @@ struct lbm_handle {
   std::vector<int> seen;                // kinds of run met so far (2 count + parity)
   double* track = nullptr;  // fused volume output (device address), or null
   int64_t track_slots = 1;  // steps of volume history in `track`
-  bool tma_ok = false;      // every case allows the bulk-copy kernel
-  int kernel = 0;           // 0 auto, 1 register-pipelined, 2 bulk-copy staged
+  bool tma_ok = false;      // every case allows the staged kernel
+  int kernel = 0;           // 0 auto, 1 register-pipelined, 2 staged, 3 one launch for many steps
   long long wait_cycles = lbmk::kWaitCycles;  // bound of the device waits
   // device pointers
   int32_t* flags = nullptr;

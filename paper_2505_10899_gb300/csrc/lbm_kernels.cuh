@@ -239,7 +239,7 @@ __device__ __forceinline__ void step_item(const StepArgs<T>& a, int item, Ring<T
   };
   // write phi/psi of local row k (k >= -1) into the ring.  phi is the plain
   // sum of the nine pulled values (FP32: the low part of g_0 enters only the
-  // rest-population update, as in the bulk-copy kernel)
+  // rest-population update, as in the staged kernel)
   auto put_row = [&](int k, const T G[9], const T H[9]) {
     const int s = (k + 4) & 3;
     if (act) {
